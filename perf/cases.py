@@ -25,6 +25,7 @@ from paper_1411_4439_gb300 import autograd as A
 FAT, NAIK = 0.9, -1.0 / 24.0
 PRECS = {"f64": H.HISQ_F64, "f32": H.HISQ_F32, "f16": H.HISQ_F16}
 REAL_BYTES = {"f64": 8, "f32": 4, "f16": 2}
+ROWS = [1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16]   # bundle sizes the per-rhs layouts take
 CHUNK = {"f32": 2, "f16": 4}               # rhs in a 16-byte chunk of the bundle layout
 OPS = {"M": H.HISQ_OP_M, "Mdag": H.HISQ_OP_MDAG, "dM": H.HISQ_OP_DM_DMU, "d2M": H.HISQ_OP_D2M_DMU2}
 FLOPS = 1146                               # of one Dslash, per output site and rhs
@@ -88,7 +89,7 @@ def draw(rng):
         layout = rng.choice(["bundle", "bundle", "aos", "soa"])
         if layout != "bundle" and rng.random() < 0.4:
             prec, ru, rn = "f64", 18, 18
-        n = rng.choice([4, 8, 12, 16]) if layout == "bundle" else rng.randint(1, 16)
+        n = rng.choice([4, 8, 12, 16] if layout == "bundle" else ROWS)
         top = 8_000_000 * (4 if prec != "f64" else 1) // n
         return dict(kind=kind, prec=prec, layout=layout, L=_draw_lattice(rng, 4096, min(64 ** 3 * 16, top)), n=n, ru=ru,
                     rn=rn, mu=rng.choice([0.0, 0.0, 0.1]), parity=rng.randint(0, 1), source=source)
@@ -110,7 +111,7 @@ def draw(rng):
         return dict(kind=kind, prec="f64", L=_draw_lattice(rng, 4096, 65536), n=rng.randint(1, 4), ru=18, rn=18,
                     mass=round(rng.uniform(0.05, 0.15), 3), mu=round(rng.uniform(0.0, 0.15), 3), source=source)
     if kind == "mdagm":
-        n = rng.randint(1, 12)
+        n = rng.choice([k for k in ROWS if k <= 12])
         return dict(kind=kind, prec=prec, L=_draw_lattice(rng, 4096, 8_000_000 // n), n=n, ru=ru, rn=rn,
                     mass=round(rng.uniform(0.002, 0.1), 4), source=source)
     if kind == "apply":
