@@ -109,7 +109,9 @@ const char* hisq_last_error(void);
  * hisq_gauge_load packs U and N into the internal site-major SoA layout
  * [parity][mu][complex component][V_h] in precision `prec`, and always also
  * keeps an FP64 R18 copy used by FP64 Dslash calls and by the CG's FP64
- * reliable updates. prec == HISQ_F64 requires R18 for both fields.
+ * reliable updates (as 55-bit fixed point with one exponent per field and
+ * direction where all links of a direction are of similar size, else doubles;
+ * FP64 Dslash results carry no larger rounding error from the former). prec == HISQ_F64 requires R18 for both fields.
  * prec == HISQ_F16 stores every link real as a 16-bit integer q with value
  * q * s_c, one scale s_c = max |Re|,|Im| / 32767 per stored complex
  * component c of each field (2^-15 of the range, where IEEE half keeps only

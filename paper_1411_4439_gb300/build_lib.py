@@ -101,8 +101,13 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
         dflags += [f"-DHISQ_FAMILY={name}_bundle", f"-DHISQ_BUNDLE_FULL={full}"]
         tasks.append(([nvcc, *ARCH, *NVFLAGS, *dflags, "-c", os.path.join(CSRC, "dslash_bundle_inst.cu"),
                        "-o", obj], obj))
+    for layout, suffix in ((0, "aos"), (1, "soa")):
+        obj = os.path.join(BUILD, f"dslash_fx64_{suffix}.o")
+        dflags = [f"-DHISQ_FAMILY=dslash_fx64_{suffix}", f"-DHISQ_LAYOUT={layout}"]
+        tasks.append(([nvcc, *ARCH, *NVFLAGS, *dflags, "-c", os.path.join(CSRC, "dslash_fx64_inst.cu"),
+                       "-o", obj], obj))
     # longest compiles first
-    tasks.sort(key=lambda t: 0 if "_bundle.o" in t[1] else 1)
+    tasks.sort(key=lambda t: 0 if "_bundle.o" in t[1] or "_fx64_" in t[1] else 1)
     jobs = jobs or min(len(tasks), max(1, os.cpu_count() or 1))
     with cf.ThreadPoolExecutor(max_workers=jobs) as ex:
         objs = list(ex.map(_compile, tasks))

@@ -24,6 +24,10 @@ HISQ_FAMILY_DECL(dslash_f16_12_14);
 HISQ_FAMILY_DECL(dslash_f16_14_14);
 #undef HISQ_FAMILY_DECL
 
+// FP64 on fixed-point links (dslash_fx64_inst.cu); split: lanes per site
+cudaError_t dslash_fx64_aos(const DslashArgs&, int epi, int rpt, int split, cudaStream_t);
+cudaError_t dslash_fx64_soa(const DslashArgs&, int epi, int rpt, int split, cudaStream_t);
+
 // bundle-layout families (dslash_bundle_inst.cu)
 cudaError_t dslash_f32_18_18_bundle(const DslashArgs&, int, int, int, int, cudaStream_t);
 cudaError_t dslash_f32_18_14_bundle(const DslashArgs&, int, int, int, int, cudaStream_t);
@@ -165,6 +169,15 @@ static cudaError_t launch_bundle(const DslashArgs& a, int prec, int ru, int rn, 
     return cudaErrorInvalidValue;
 }
 
+// Lanes per site of the fixed-point FP64 kernel: the four directions of a site
+// on four lanes while one lane per site would leave schedulers without a warp
+// (8^4, n = 1: 14.7 us with one lane, 8.3 with four; 16^4, n = 1, where every
+// scheduler has one or two: 24.6 and 31).
+static int fx64_split(const DslashArgs& a, int rpt) {
+    const long long warps = ((long long)a.g.vh * (a.nrhs / rpt) + 31) / 32;
+    return rpt <= 2 && warps < 4ll * device_sm_count() ? 4 : 1;
+}
+
 cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi,
                           const DslashTune& t, cudaStream_t s) {
     if (!dslash_variant_supported(prec, ru, rn, epi)) return cudaErrorInvalidValue;
@@ -181,6 +194,10 @@ cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi
         return launch_dslash(c, prec, ru, rn, epi, t, s);
     }
     const int r = t.rpt, b = t.minb, k = t.kind, l = t.layout;
+    if (prec == HISQ_F64 && a.fx) {
+        const int split = fx64_split(a, r);
+        return l == HISQ_SOA ? dslash_fx64_soa(a, epi, r, split, s) : dslash_fx64_aos(a, epi, r, split, s);
+    }
     if (prec == HISQ_F64) return dslash_f64_18_18(a, epi, r, b, k, l, s);
     const int key = ru * 100 + rn;
     if (prec == HISQ_F32) {

@@ -135,6 +135,61 @@ __device__ __forceinline__ short2 store_comp<short2>(double2 v, const double* co
     return make_short2(quantize(v.x, inv), quantize(v.y, inv));
 }
 
+// fixed-point FP64 storage: v * scale as an integer of at most 55 bits, split
+// into limbs of 28 bits (low limb balanced, see dslash_fx64.cuh)
+__device__ __forceinline__ int2 fx_split(double v, double scale) {
+    const long long q = __double2ll_rn(v * scale);
+    const int lo = (int)((unsigned)q << 4) >> 4;
+    return make_int2((int)((q - lo) >> 28), lo);
+}
+
+__global__ void pack_fx_kernel(Geom g, const double2* __restrict__ canon, const double* __restrict__ scale,
+                               int4* __restrict__ out) {
+    const long long V = 2ll * g.vh;
+    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
+         w += (long long)gridDim.x * blockDim.x) {
+        const int mu = (int)(w / V);
+        const Site s = site_of(g, w - mu * V);
+        const double sc = scale[mu];
+        int4* block = out + (size_t)(s.parity * 4 + mu) * 9 * g.vh;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const double2 v = canon[w * 9 + c];
+            const int2 re = fx_split(v.x, sc), im = fx_split(v.y, sc);
+            block[(size_t)c * g.vh + s.h] = make_int4(re.x, re.y, im.x, im.y);
+        }
+    }
+}
+
+// blockIdx.y = mu; range preset by the launcher
+__global__ void __launch_bounds__(256) range_kernel(Geom g, const double2* __restrict__ canon,
+                                                    unsigned long long* range) {
+    const long long V = 2ll * g.vh;
+    const int mu = blockIdx.y;
+    const double inf = __longlong_as_double(0x7ff0000000000000ll);
+    double hi = 0.0, lo = inf;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
+        const double2* m = canon + (mu * V + i) * 9;
+        double mx = 0.0;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const double2 v = m[c];
+            const double a = fabs(v.x), b = fabs(v.y);
+            mx = (a <= inf && b <= inf) ? fmax(mx, fmax(a, b)) : inf;   // NaN -> inf
+        }
+        hi = fmax(hi, mx);
+        if (mx > 0.0) lo = fmin(lo, mx);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(range + mu, (unsigned long long)__double_as_longlong(hi));
+        atomicMin(range + 4 + mu, (unsigned long long)__double_as_longlong(lo));
+    }
+}
+
 template <typename C>
 __global__ void pack_kernel(Geom g, const double2* __restrict__ canon, int recon, int hop,
                             double inv_s, C* __restrict__ out, unsigned long long* err_bits,
@@ -260,6 +315,22 @@ cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int
             break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_link_range(const Geom& g, const double2* canon, unsigned long long* range, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(range, 0, 4 * sizeof(*range), s);
+    // 0x7f7f..: a finite double above any other link maximum that counts
+    if (e == cudaSuccess) e = cudaMemsetAsync(range + 4, 0x7f, 4 * sizeof(*range), s);
+    if (e != cudaSuccess) return e;
+    const unsigned b = (grid_for(2ll * g.vh) + 3) / 4;
+    range_kernel<<<dim3(b, 4), 256, 0, s>>>(g, canon, range);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_links_fx(const Geom& g, const double2* canon, const double* scale, void* out,
+                                 cudaStream_t s) {
+    pack_fx_kernel<<<grid_for(8ll * g.vh), 256, 0, s>>>(g, canon, scale, (int4*)out);
     return cudaGetLastError();
 }
 

@@ -183,8 +183,10 @@ struct hisq_gauge_s {
     float lscale_n[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
     void* U_lo = nullptr;        // storage copy (prec, recon)
     void* N_lo = nullptr;
-    double2* U64 = nullptr;      // FP64 R18 copy
+    double2* U64 = nullptr;      // FP64 R18 copy: doubles, or with fx int4 limbs (dslash_fx64.cuh)
     double2* N64 = nullptr;
+    int fx = 0;
+    int fx_exp[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     size_t link_bytes = 0;
     int tune_rpt = 0;            // 0 = automatic
     int tune_minb = 0;
@@ -254,6 +256,51 @@ hisq_status pack_field(hisq_gauge g, const double2* canon, int prec, int recon, 
     if (!(err <= recon_tol))
         return fail(HISQ_ERECON, "%s links are not representable with %d reals: max reconstruct error %.3e > tol %.3e",
                     name, recon, err, recon_tol);
+    return HISQ_OK;
+}
+
+// Whether the FP64 links go into fixed point, and their block exponents: in
+// every (field, direction) all links finite and every nonzero link's largest
+// real within a factor of 16 of the block's largest, so that the smallest
+// links still carry 51 bits (Haar links x a constant lie within 2.5).
+hisq_status choose_fx(hisq_gauge g, const double2* cu, const double2* cn, cudaStream_t s) {
+    unsigned long long* range = nullptr;
+    HISQ_CUDA(cudaMalloc(&range, 16 * sizeof(unsigned long long)));
+    unsigned long long bits[16] = {0};
+    cudaError_t e = launch_link_range(g->g, cu, range, s);
+    if (e == cudaSuccess) e = launch_link_range(g->g, cn, range + 8, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(bits, range, sizeof(bits), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(range);
+    HISQ_CUDA(e);
+    g->fx = 1;
+    for (int f = 0; f < 2; ++f)
+        for (int mu = 0; mu < 4; ++mu) {
+            double hi, lo;
+            memcpy(&hi, &bits[8 * f + mu], sizeof(hi));
+            memcpy(&lo, &bits[8 * f + 4 + mu], sizeof(lo));
+            int ex = 0;
+            if (hi > 0.0 && std::isfinite(hi)) std::frexp(hi, &ex);
+            g->fx_exp[4 * f + mu] = ex;
+            if (!std::isfinite(hi) || (hi > 0.0 && !(lo >= hi / 16.0)) || ex < -200 || ex > 200) g->fx = 0;
+        }
+    return HISQ_OK;
+}
+
+hisq_status pack_field_fx(hisq_gauge g, const double2* canon, int field, double2** out, size_t* bytes,
+                          cudaStream_t s) {
+    const size_t sz = 2 * 4 * 9 * (size_t)g->g.vh * sizeof(double2);
+    HISQ_CUDA(cudaMalloc(out, sz));
+    *bytes += sz;
+    double sc[4];
+    for (int mu = 0; mu < 4; ++mu) sc[mu] = std::ldexp(1.0, 55 - g->fx_exp[4 * field + mu]);
+    double* scale = nullptr;
+    HISQ_CUDA(cudaMalloc(&scale, sizeof(sc)));
+    cudaError_t e = cudaMemcpyAsync(scale, sc, sizeof(sc), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_pack_links_fx(g->g, canon, scale, *out, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(scale);
+    HISQ_CUDA(e);
     return HISQ_OK;
 }
 
@@ -333,8 +380,14 @@ extern "C" hisq_status hisq_gauge_load(const int L[4], const void* U, const void
         g->r12_inv_scale = 1.0 / sc;
     }
     size_t bytes = 0;
-    st = pack_field(g, cu, HISQ_F64, 18, 1, recon_tol, (void**)&g->U64, &bytes, "fat", s);
-    if (st == HISQ_OK) st = pack_field(g, cn, HISQ_F64, 18, 3, recon_tol, (void**)&g->N64, &bytes, "Naik", s);
+    st = choose_fx(g, cu, cn, s);
+    if (st == HISQ_OK && g->fx) {
+        st = pack_field_fx(g, cu, 0, &g->U64, &bytes, s);
+        if (st == HISQ_OK) st = pack_field_fx(g, cn, 1, &g->N64, &bytes, s);
+    } else if (st == HISQ_OK) {
+        st = pack_field(g, cu, HISQ_F64, 18, 1, recon_tol, (void**)&g->U64, &bytes, "fat", s);
+        if (st == HISQ_OK) st = pack_field(g, cn, HISQ_F64, 18, 3, recon_tol, (void**)&g->N64, &bytes, "Naik", s);
+    }
     if (st == HISQ_OK) {
         if (prec == HISQ_F64) {
             g->U_lo = g->U64;
@@ -463,6 +516,14 @@ namespace {
 int link_recon_u(hisq_gauge g, int prec) { return prec == HISQ_F64 ? 18 : g->recon_U; }
 int link_recon_n(hisq_gauge g, int prec) { return prec == HISQ_F64 ? 18 : g->recon_N; }
 
+// rhs per thread of the fixed-point FP64 kernel: two share the link loads once
+// the threads fill the SMs one and a half times over at 12 warps each (48^3x12,
+// n = 8: 1.89 ms against 2.06 with one), else one, for more warps in flight
+// (16^4, n = 4: 58 us against 66).
+int auto_rpt_fx64(hisq_gauge g, int n) {
+    return n % 2 == 0 && (long long)g->g.vh * (n / 2) >= 18ll * 32 * device_sm_count() ? 2 : n > 8 ? 2 : 1;
+}
+
 int auto_rpt(int n, int prec) {
     const int mx = dslash_max_rpt(prec);
     int r = 1;
@@ -545,7 +606,8 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
         if (it != g->tuned.end()) return it->second;
     }
     int r = requested ? requested : g->tune_rpt;
-    if (r == 0 || r > dslash_max_rpt(prec) || n % r != 0 || n / r > 8) r = auto_rpt(n, prec);
+    if (r == 0 || r > dslash_max_rpt(prec) || n % r != 0 || n / r > 8)
+        r = prec == HISQ_F64 && g->fx ? auto_rpt_fx64(g, n) : auto_rpt(n, prec);
     DslashTune t = dslash_default_tune(prec, r, layout);
     const int kind = kind_of_flags(g->tune_flags);
     if (!requested && g->tune_minb && r == g->tune_rpt && dslash_mapping_built(prec, r, g->tune_minb, kind) &&
@@ -601,6 +663,8 @@ void fill_common(DslashArgs& a, hisq_gauge g, int prec, int parity, int n) {
         a.lscale_u[c] = g->lscale_u[c];
         a.lscale_n[c] = g->lscale_n[c];
     }
+    a.fx = prec == HISQ_F64 ? g->fx : 0;
+    for (int c = 0; c < 8; ++c) a.fx_exp[c] = g->fx_exp[c];
     a.red_mode = RED_NONE;
     a.finish = FIN_STORE;
 }

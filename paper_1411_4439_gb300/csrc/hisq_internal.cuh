@@ -224,6 +224,10 @@ struct DslashArgs {
     int t_only;                         // 1: temporal hops only (d D / d mu)
     int l2_prefetch;                    // 1: bulk-prefetch each tile's links into L2
     int* status;                        // bounded waits that give up OR kFlagTimeout here (or null)
+    int fx;                             // 1: FP64 links in fixed point (dslash_fx64.cuh)
+    int fx_exp[8];                      // their block exponents, [U, N][direction]
+    int fx_f1[4], fx_f0[4], fx_fe[4];   // temporal factors (ft1, bt1, ft3, bt3) in limbs, set by the launcher
+    int fx_slow;                        // 1: a factor is out of range, FP64 arithmetic (set by the launcher)
     double r12_inv_scale;               // 1 / s for R12 fat links
     float lscale_u[9];                  // per-component scales of 16-bit fat links
     float lscale_n[9];                  // per-component scales of 16-bit Naik links
@@ -305,6 +309,16 @@ cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int
 // field, as the bits of non-negative doubles OR-maximised into maxbits[c].
 cudaError_t launch_link_absmax(const Geom& g, const double2* canon, int recon, int hop,
                                double r12_inv_scale, unsigned long long* maxbits, cudaStream_t s);
+// Range of the links of a field, per direction mu: the bits of the largest
+// |Re|, |Im| into range[mu] (+inf if any is not finite) and of the smallest
+// over nonzero links of a link's largest into range[4 + mu] (+inf if none).
+// range: 8 device values, set by the call.
+cudaError_t launch_link_range(const Geom& g, const double2* canon, unsigned long long* range, cudaStream_t s);
+// Pack canonical links into the fixed-point FP64 storage (dslash_fx64.cuh):
+// R18 components as int4 limbs (re1, re0, im1, im0) of value * scale[mu],
+// scale (device) = 2^(55 - e) of each direction.
+cudaError_t launch_pack_links_fx(const Geom& g, const double2* canon, const double* scale, void* out,
+                                 cudaStream_t s);
 // Compress to double [4][V][r] and back (ABI helpers).
 cudaError_t launch_compress_links(const Geom& g, const double2* canon, int recon, int hop,
                                   double r12_inv_scale, double* packed,
