@@ -38,15 +38,15 @@ struct Site {
     int x, y, z, t, parity, h;
 };
 
-__device__ __forceinline__ Site site_of(const Geom& g, long long i) {
+__device__ __forceinline__ Site site_of(const Geom& g, unsigned i) {   // i < V <= 2^27
     Site s;
-    long long r = i;
-    s.x = (int)(r % g.L[0]);
-    r /= g.L[0];
-    s.y = (int)(r % g.L[1]);
-    r /= g.L[1];
-    s.z = (int)(r % g.L[2]);
-    s.t = (int)(r / g.L[2]);
+    unsigned r = i;
+    s.x = (int)(r % (unsigned)g.L[0]);
+    r /= (unsigned)g.L[0];
+    s.y = (int)(r % (unsigned)g.L[1]);
+    r /= (unsigned)g.L[1];
+    s.z = (int)(r % (unsigned)g.L[2]);
+    s.t = (int)(r / (unsigned)g.L[2]);
     s.parity = (s.x + s.y + s.z + s.t) & 1;
     s.h = (int)(i >> 1);
     return s;
@@ -103,137 +103,210 @@ __device__ __forceinline__ double encode(const double2* m, int recon, int sign, 
     return err;
 }
 
-template <typename C> __device__ __forceinline__ C narrow(double2 v);
-template <> __device__ __forceinline__ double2 narrow<double2>(double2 v) { return v; }
-template <> __device__ __forceinline__ float2 narrow<float2>(double2 v) {
-    return make_float2((float)v.x, (float)v.y);
-}
-template <> __device__ __forceinline__ __half2 narrow<__half2>(double2 v) {
-    return __floats2half2_rn((float)v.x, (float)v.y);
-}
-
 __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* bits, double v) {
     if (!(v >= 0.0)) v = __longlong_as_double(0x7ff0000000000000ll);   // NaN -> +inf
     atomicMax(bits, (unsigned long long)__double_as_longlong(v));
 }
 
-// 16-bit fixed point: round to nearest of v / scale, clamped to +-32767
-__device__ __forceinline__ short quantize(double v, double inv_scale) {
-    double q = rint(v * inv_scale);
-    q = fmin(fmax(q, -32767.0), 32767.0);
-    return (short)q;
+// bits of |v|: as unsigned integers they order like the values (NaN above
+// infinity), and the ALU compares them 30 times faster than the FP64 pipe
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
+    return a > b ? a : b;
 }
 
-template <typename C>
-__device__ __forceinline__ C store_comp(double2 v, const double* comp_scale, int c) {
-    return narrow<C>(v);
-}
-template <>
-__device__ __forceinline__ short2 store_comp<short2>(double2 v, const double* comp_scale, int c) {
-    const double sc = comp_scale[c];
-    const double inv = sc > 0.0 ? 1.0 / sc : 0.0;
-    return make_short2(quantize(v.x, inv), quantize(v.y, inv));
+// Stored component 6 of an R14 link (z = row3_k / conj(row1 x row2)_k for the
+// largest k) or the factor of row 3 of an R12 one, and the largest deviation
+// of row 3 = f conj(row1 x row2) from the input.
+template <int RECON>
+__device__ __forceinline__ double2 third_factor(const double2* m, int sign, double inv_s, double& err) {
+    double2 cc[3];
+    cross_conj(m, cc);
+    double2 f;
+    if (RECON == 14) {
+        double n2[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) n2[c] = cc[c].x * cc[c].x + cc[c].y * cc[c].y;
+        double2 ck = cc[0], mk = m[6];
+        double d = n2[0];
+        if (n2[1] > d) { ck = cc[1]; mk = m[7]; d = n2[1]; }
+        if (n2[2] > d) { ck = cc[2]; mk = m[8]; d = n2[2]; }
+        f = make_double2(0.0, 0.0);
+        if (d > 0.0) {
+            const double inv = 1.0 / d;
+            f = make_double2((mk.x * ck.x + mk.y * ck.y) * inv, (mk.y * ck.x - mk.x * ck.y) * inv);
+        }
+    } else {
+        f = make_double2(sign > 0 ? inv_s : -inv_s, 0.0);
+    }
+    double e2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double2 dv = zsub(zmul(f, cc[c]), m[6 + c]);
+        e2 = fmax(e2, dv.x * dv.x + dv.y * dv.y);
+    }
+    err = fmax(err, sqrt(e2));
+    return f;
 }
 
-// fixed-point FP64 storage: v * scale as an integer of at most 55 bits, split
-// into limbs of 28 bits (low limb balanced, see dslash_fx64.cuh)
-__device__ __forceinline__ int2 fx_split(double v, double scale) {
-    const long long q = __double2ll_rn(v * scale);
+// One pass over a field before it is packed; blockIdx.y = mu. Every block
+// reduces its maxima in shared memory and issues one atomic per value; with
+// atomics from every thread the pass took 5.6 to 6.9 ms at 48^3x12, now
+// 0.19 ms (R18, 4.0 TB/s) and 1.08 ms (R14: FP64 pipe, 78 operations a link
+// for the reconstruct check).
+template <int RECON>
+__global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __restrict__ canon, int hop, double inv_s,
+                                                   LinkScan* out) {
+    constexpr int NC = RECON / 2;
+    const unsigned V = 2u * (unsigned)g.vh;
+    const int mu = blockIdx.y;
+    unsigned long long mx[NC], hi = 0ull, lo = ~0ull;
+    double err = 0.0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) mx[c] = 0ull;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const double2* src = canon + ((size_t)mu * V + i) * 9;
+        double2 m[9];
+        unsigned long long link = 0ull;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            m[c] = src[c];
+            const unsigned long long b = umax64(abs_bits(m[c].x), abs_bits(m[c].y));
+            if (c < NC && (c < 6 || RECON == 18)) mx[c] = umax64(mx[c], b);
+            link = umax64(link, b);
+        }
+        hi = umax64(hi, link);
+        if (link != 0ull && link < lo) lo = link;
+        if (RECON != 18) {
+            const int sg = RECON == 12 ? staggered_sign(g, site_of(g, i), mu, hop) : 1;
+            const double2 f = third_factor<RECON>(m, sg, inv_s, err);
+            if (RECON == 14) mx[NC - 1] = umax64(mx[NC - 1], umax64(abs_bits(f.x), abs_bits(f.y)));
+        }
+    }
+    __shared__ unsigned long long s_v[12][8];
+    unsigned long long v[12];
+#pragma unroll
+    for (int c = 0; c < 9; ++c) v[c] = c < NC ? mx[c < NC ? c : 0] : 0ull;
+    v[9] = hi;
+    v[10] = ~lo;   // the smallest as a largest
+    v[11] = (unsigned long long)__double_as_longlong(err);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        for (int o = 16; o > 0; o >>= 1) v[c] = umax64(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
+        if (lane == 0) s_v[c][warp] = v[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 12) {
+        unsigned long long t = 0ull;
+        for (int w = 0; w < 8; ++w) t = umax64(t, s_v[threadIdx.x][w]);
+        const int c = threadIdx.x;
+        if (t != 0ull)
+            atomicMax(c < 9 ? &out->comp[c] : c == 9 ? &out->hi[mu] : c == 10 ? &out->nlo[mu] : &out->err, t);
+    }
+}
+
+// Component 6 of an R14 link alone: the pivot k is chosen in FP32 (where two
+// of the |cc_k| agree to FP32 rounding either serves), the rest as in
+// third_factor; 26 FP64 operations instead of 78.
+__device__ __forceinline__ double2 r14_factor(const double2* m) {
+    float2 u[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) u[c] = make_float2((float)m[c].x, (float)m[c].y);
+    auto cross2 = [&](int a, int b, int c, int d) {
+        const float x = u[a].x * u[b].x - u[a].y * u[b].y - (u[c].x * u[d].x - u[c].y * u[d].y);
+        const float y = u[a].x * u[b].y + u[a].y * u[b].x - (u[c].x * u[d].y + u[c].y * u[d].x);
+        return x * x + y * y;
+    };
+    const float n0 = cross2(1, 5, 2, 4), n1 = cross2(2, 3, 0, 5), n2 = cross2(0, 4, 1, 3);
+    const int k = (n1 > n0) ? (n2 > n1 ? 2 : 1) : (n2 > n0 ? 2 : 0);
+    const float best = fmaxf(n0, fmaxf(n1, n2));
+    if (!(best > 1e-30f && best < 1e30f)) {   // FP32 range left
+        double unused = 0.0;
+        return third_factor<14>(m, 1, 1.0, unused);
+    }
+    const double2 a = k == 0 ? m[1] : k == 1 ? m[2] : m[0], b = k == 0 ? m[5] : k == 1 ? m[3] : m[4];
+    const double2 c = k == 0 ? m[2] : k == 1 ? m[0] : m[1], d = k == 0 ? m[4] : k == 1 ? m[5] : m[3];
+    const double2 mk = k == 0 ? m[6] : k == 1 ? m[7] : m[8];
+    const double2 ck = zconj(zsub(zmul(a, b), zmul(c, d)));
+    const double inv = 1.0 / (ck.x * ck.x + ck.y * ck.y);
+    return make_double2((mk.x * ck.x + mk.y * ck.y) * inv, (mk.y * ck.x - mk.x * ck.y) * inv);
+}
+
+// fixed-point FP64 storage: v 2^(55 - e) rounded to an integer of at most 55
+// bits, split into limbs of 28 bits (low limb balanced, see dslash_fx64.cuh),
+// with integer instructions (|v| < 2^e, so the mantissa moves right)
+__device__ __forceinline__ int2 fx_split(double v, int e) {
+    const unsigned long long bits = abs_bits(v);
+    const int field = (int)(bits >> 52);
+    // left-aligned mantissa; bits to drop: 64 - 55 - (field - 1022) + e >= 9
+    const unsigned long long m = (bits << 11) | 0x8000000000000000ull;
+    const int sh = 9 + e + 1022 - field;
+    long long q = 0;
+    if (field > 0 && sh <= 63) q = (long long)((m >> sh) + ((m >> (sh - 1)) & 1ull));
+    q = __double_as_longlong(v) < 0 ? -q : q;
     const int lo = (int)((unsigned)q << 4) >> 4;
     return make_int2((int)((q - lo) >> 28), lo);
 }
 
-__global__ void pack_fx_kernel(Geom g, const double2* __restrict__ canon, const double* __restrict__ scale,
-                               int4* __restrict__ out) {
-    const long long V = 2ll * g.vh;
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
-         w += (long long)gridDim.x * blockDim.x) {
-        const int mu = (int)(w / V);
-        const Site s = site_of(g, w - mu * V);
-        const double sc = scale[mu];
-        int4* block = out + (size_t)(s.parity * 4 + mu) * 9 * g.vh;
-#pragma unroll
-        for (int c = 0; c < 9; ++c) {
-            const double2 v = canon[w * 9 + c];
-            const int2 re = fx_split(v.x, sc), im = fx_split(v.y, sc);
-            block[(size_t)c * g.vh + s.h] = make_int4(re.x, re.y, im.x, im.y);
-        }
-    }
+// 16-bit fixed point: round to nearest of v / scale, clamped to +-32767
+__device__ __forceinline__ short quantize(double v, double inv_scale) {
+    const int q = __double2int_rn(v * inv_scale);
+    return (short)min(max(q, -32767), 32767);
+}
+__device__ __forceinline__ float4 store_pair(double2 a, double2 b, const double*, int, float2) {
+    return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+}
+__device__ __forceinline__ short4 store_pair(double2 a, double2 b, const double* inv, int c, short2) {
+    return make_short4(quantize(a.x, inv[c]), quantize(a.y, inv[c]), quantize(b.x, inv[c + 1]), quantize(b.y, inv[c + 1]));
+}
+__device__ __forceinline__ float2 store_one(double2 a, const double*, int, float2) {
+    return make_float2((float)a.x, (float)a.y);
+}
+__device__ __forceinline__ short2 store_one(double2 a, const double* inv, int c, short2) {
+    return make_short2(quantize(a.x, inv[c]), quantize(a.y, inv[c]));
 }
 
-// blockIdx.y = mu; range preset by the launcher
-__global__ void __launch_bounds__(256) range_kernel(Geom g, const double2* __restrict__ canon,
-                                                    unsigned long long* range) {
-    const long long V = 2ll * g.vh;
+// One pass over a field writes its FP64 copy (fixed point or doubles) and,
+// unless the storage precision is FP64 (LC = double2), the storage copy. At
+// 48^3x12 with 16-bit storage 0.52 ms (R18, 1.7 GB) and 0.78 ms (R14), where
+// separate passes took 1.87 and 2.92 ms; the FP64 pipe bounds it (the
+// quantisation multiplies, z), so the fixed-point split uses integers only.
+template <typename LC, int RECON>
+__global__ void __launch_bounds__(256) pack_kernel(Geom g, const double2* __restrict__ canon, int fx, LinkScales sc,
+                                                   double2* __restrict__ out64, LC* __restrict__ out_lo) {
+    constexpr int NC = RECON / 2;
+    const unsigned V = 2u * (unsigned)g.vh;
     const int mu = blockIdx.y;
-    const double inf = __longlong_as_double(0x7ff0000000000000ll);
-    double hi = 0.0, lo = inf;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
-        const double2* m = canon + (mu * V + i) * 9;
-        double mx = 0.0;
+    const int fxe = sc.fx_exp[mu];
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
+        const double2* src = canon + ((size_t)mu * V + i) * 9;
+        const Site s = site_of(g, i);
+        double2 m[9];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) m[c] = src[c];
+        double2* o64 = out64 + (size_t)(s.parity * 4 + mu) * 9 * g.vh + s.h;
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
-            const double2 v = m[c];
-            const double a = fabs(v.x), b = fabs(v.y);
-            mx = (a <= inf && b <= inf) ? fmax(mx, fmax(a, b)) : inf;   // NaN -> inf
+            if (fx) {
+                const int2 re = fx_split(m[c].x, fxe), im = fx_split(m[c].y, fxe);
+                reinterpret_cast<int4*>(o64)[(size_t)c * g.vh] = make_int4(re.x, re.y, im.x, im.y);
+            } else {
+                o64[(size_t)c * g.vh] = m[c];
+            }
         }
-        hi = fmax(hi, mx);
-        if (mx > 0.0) lo = fmin(lo, mx);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(range + mu, (unsigned long long)__double_as_longlong(hi));
-        atomicMin(range + 4 + mu, (unsigned long long)__double_as_longlong(lo));
-    }
-}
-
-template <typename C>
-__global__ void pack_kernel(Geom g, const double2* __restrict__ canon, int recon, int hop,
-                            double inv_s, C* __restrict__ out, unsigned long long* err_bits,
-                            const double* __restrict__ comp_scale) {
-    const int nc = recon / 2;
-    const long long V = 2ll * g.vh;
-    double worst = 0.0;
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
-         w += (long long)gridDim.x * blockDim.x) {
-        const int mu = (int)(w / V);
-        const long long i = w - mu * V;
-        const Site s = site_of(g, i);
-        double2 m[9], enc[9];
+        if constexpr (LinkPair<LC>::paired) {
+            if (RECON == 14) m[6] = r14_factor(m);
+            using P = typename LinkPair<LC>::V;
+            LC* block = out_lo + (size_t)(s.parity * 4 + mu) * NC * g.vh;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) m[c] = canon[w * 9 + c];
-        const int sg = (recon == 12) ? staggered_sign(g, s, mu, hop) : 1;
-        worst = fmax(worst, encode(m, recon, sg, inv_s, enc));
-        C* block = out + ((size_t)(s.parity * 4 + mu) * nc) * g.vh;
-        for (int c = 0; c < nc; ++c) block[link_offset<C>(c, nc, g.vh, s.h)] = store_comp<C>(enc[c], comp_scale, c);
+            for (int p = 0; p < NC / 2; ++p)
+                reinterpret_cast<P*>(block)[(size_t)p * g.vh + s.h] = store_pair(m[2 * p], m[2 * p + 1], sc.inv, 2 * p, LC{});
+            if constexpr (NC & 1) block[(size_t)(NC - 1) * g.vh + s.h] = store_one(m[NC - 1], sc.inv, NC - 1, LC{});
+        }
     }
-    if (err_bits != nullptr) atomic_max_nonneg(err_bits, worst);
-}
-
-__global__ void absmax_kernel(Geom g, const double2* __restrict__ canon, int recon, int hop,
-                              double inv_s, unsigned long long* maxbits) {
-    const int nc = recon / 2;
-    const long long V = 2ll * g.vh;
-    double mx[9];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) mx[c] = 0.0;
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
-         w += (long long)gridDim.x * blockDim.x) {
-        const int mu = (int)(w / V);
-        const Site s = site_of(g, w - mu * V);
-        double2 m[9], enc[9];
-#pragma unroll
-        for (int c = 0; c < 9; ++c) m[c] = canon[w * 9 + c];
-        const int sg = (recon == 12) ? staggered_sign(g, s, mu, hop) : 1;
-        encode(m, recon, sg, inv_s, enc);
-#pragma unroll
-        for (int c = 0; c < 9; ++c)
-            if (c < nc) mx[c] = fmax(mx[c], fmax(fabs(enc[c].x), fabs(enc[c].y)));
-    }
-    for (int c = 0; c < nc; ++c) atomic_max_nonneg(maxbits + c, mx[c]);
 }
 
 __global__ void compress_kernel(Geom g, const double2* __restrict__ canon, int recon, int hop,
@@ -245,7 +318,7 @@ __global__ void compress_kernel(Geom g, const double2* __restrict__ canon, int r
     for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
          w += (long long)gridDim.x * blockDim.x) {
         const int mu = (int)(w / V);
-        const Site s = site_of(g, w - mu * V);
+        const Site s = site_of(g, (unsigned)(w - mu * V));
         double2 m[9], enc[9];
 #pragma unroll
         for (int c = 0; c < 9; ++c) m[c] = canon[w * 9 + c];
@@ -266,7 +339,7 @@ __global__ void reconstruct_kernel(Geom g, const double* __restrict__ packed, in
     for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < 4 * V;
          w += (long long)gridDim.x * blockDim.x) {
         const int mu = (int)(w / V);
-        const Site s = site_of(g, w - mu * V);
+        const Site s = site_of(g, (unsigned)(w - mu * V));
         double2 m[9];
         for (int c = 0; c < nc; ++c)
             m[c] = make_double2(packed[w * recon + 2 * c], packed[w * recon + 2 * c + 1]);
@@ -285,9 +358,9 @@ __global__ void reconstruct_kernel(Geom g, const double* __restrict__ packed, in
     }
 }
 
-unsigned grid_for(long long work) {
+unsigned grid_for(long long work, int per_sm = 32) {
     long long b = (work + 255) / 256;
-    const long long cap = 32ll * device_sm_count();
+    const long long cap = (long long)per_sm * device_sm_count();
     if (b > cap) b = cap;
     if (b < 1) b = 1;
     return (unsigned)b;
@@ -295,48 +368,36 @@ unsigned grid_for(long long work) {
 
 }  // namespace
 
-cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, int hop,
-                              double r12_inv_scale, void* out, unsigned long long* err_bits,
-                              const double* comp_scale, cudaStream_t s) {
-    const unsigned grid = grid_for(8ll * g.vh);
-    switch (prec) {
-        case HISQ_F64:
-            pack_kernel<double2><<<grid, 256, 0, s>>>(g, canon, recon, hop, r12_inv_scale,
-                                                      (double2*)out, err_bits, comp_scale);
-            break;
-        case HISQ_F32:
-            pack_kernel<float2><<<grid, 256, 0, s>>>(g, canon, recon, hop, r12_inv_scale,
-                                                     (float2*)out, err_bits, comp_scale);
-            break;
-        case HISQ_F16:
-            if (comp_scale == nullptr) return cudaErrorInvalidValue;
-            pack_kernel<short2><<<grid, 256, 0, s>>>(g, canon, recon, hop, r12_inv_scale,
-                                                     (short2*)out, err_bits, comp_scale);
-            break;
+cudaError_t launch_link_scan(const Geom& g, const double2* canon, int recon, int hop, double r12_inv_scale,
+                             LinkScan* out, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(*out), s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((grid_for(2ll * g.vh, 2) + 3) / 4, 4);
+    switch (recon) {
+        case 18: scan_kernel<18><<<grid, 256, 0, s>>>(g, canon, hop, r12_inv_scale, out); break;
+        case 14: scan_kernel<14><<<grid, 256, 0, s>>>(g, canon, hop, r12_inv_scale, out); break;
+        case 12: scan_kernel<12><<<grid, 256, 0, s>>>(g, canon, hop, r12_inv_scale, out); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_link_range(const Geom& g, const double2* canon, unsigned long long* range, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(range, 0, 4 * sizeof(*range), s);
-    // 0x7f7f..: a finite double above any other link maximum that counts
-    if (e == cudaSuccess) e = cudaMemsetAsync(range + 4, 0x7f, 4 * sizeof(*range), s);
-    if (e != cudaSuccess) return e;
-    const unsigned b = (grid_for(2ll * g.vh) + 3) / 4;
-    range_kernel<<<dim3(b, 4), 256, 0, s>>>(g, canon, range);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack_links_fx(const Geom& g, const double2* canon, const double* scale, void* out,
-                                 cudaStream_t s) {
-    pack_fx_kernel<<<grid_for(8ll * g.vh), 256, 0, s>>>(g, canon, scale, (int4*)out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_link_absmax(const Geom& g, const double2* canon, int recon, int hop,
-                               double r12_inv_scale, unsigned long long* maxbits, cudaStream_t s) {
-    absmax_kernel<<<grid_for(8ll * g.vh), 256, 0, s>>>(g, canon, recon, hop, r12_inv_scale, maxbits);
+cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, int fx, const LinkScales& sc,
+                              void* out64, void* out_lo, cudaStream_t s) {
+    const dim3 grid((grid_for(8ll * g.vh) + 3) / 4, 4);
+    double2* o = (double2*)out64;
+#define HISQ_PACK(LC, RECON) pack_kernel<LC, RECON><<<grid, 256, 0, s>>>(g, canon, fx, sc, o, (LC*)out_lo)
+    switch (prec * 100 + recon) {
+        case HISQ_F64 * 100 + 18: HISQ_PACK(double2, 18); break;
+        case HISQ_F32 * 100 + 18: HISQ_PACK(float2, 18); break;
+        case HISQ_F32 * 100 + 14: HISQ_PACK(float2, 14); break;
+        case HISQ_F32 * 100 + 12: HISQ_PACK(float2, 12); break;
+        case HISQ_F16 * 100 + 18: HISQ_PACK(short2, 18); break;
+        case HISQ_F16 * 100 + 14: HISQ_PACK(short2, 14); break;
+        case HISQ_F16 * 100 + 12: HISQ_PACK(short2, 12); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef HISQ_PACK
     return cudaGetLastError();
 }
 

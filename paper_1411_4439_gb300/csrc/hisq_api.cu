@@ -181,6 +181,7 @@ struct hisq_gauge_s {
     double r12_inv_scale = 1.0;
     float lscale_u[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};   // 16-bit link component scales
     float lscale_n[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
+    void* link_block = nullptr;  // the allocation of all link copies
     void* U_lo = nullptr;        // storage copy (prec, recon)
     void* N_lo = nullptr;
     double2* U64 = nullptr;      // FP64 R18 copy: doubles, or with fx int4 limbs (dslash_fx64.cuh)
@@ -210,107 +211,88 @@ extern "C" const char* hisq_last_error(void) { return g_last_error.c_str(); }
 // ---------------------------------------------------------------------------
 namespace {
 
-hisq_status pack_field(hisq_gauge g, const double2* canon, int prec, int recon, int hop,
-                       double recon_tol, void** out, size_t* bytes, const char* name,
-                       cudaStream_t s) {
-    const size_t nc = (size_t)recon / 2;
-    const size_t sz = 2 * 4 * nc * (size_t)g->g.vh * prec_complex_bytes(prec);
-    HISQ_CUDA(cudaMalloc(out, sz));
-    *bytes += sz;
-    // scratch: [0] reconstruct error bits, [1..9] component maxima (16-bit
-    // storage), then the 9 component scales as doubles
-    unsigned long long* scratch = nullptr;
-    HISQ_CUDA(cudaMalloc(&scratch, 19 * sizeof(unsigned long long)));
-    unsigned long long* err_bits = scratch;
-    double* comp_scale = reinterpret_cast<double*>(scratch + 10);
-    cudaError_t e = cudaMemsetAsync(scratch, 0, 19 * sizeof(unsigned long long), s);
-    if (e == cudaSuccess && prec == HISQ_F16) {
-        // one scale per stored component: its largest |Re|, |Im| / 32767
-        e = launch_link_absmax(g->g, canon, recon, hop, g->r12_inv_scale, scratch + 1, s);
-        unsigned long long mb[9] = {0};
-        if (e == cudaSuccess) e = cudaMemcpyAsync(mb, scratch + 1, sizeof(mb), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        double sc[9];
-        float* keep = (hop == 1) ? g->lscale_u : g->lscale_n;
-        for (size_t c = 0; c < 9; ++c) {
-            double mx;
-            memcpy(&mx, &mb[c], sizeof(mx));
-            sc[c] = (c < nc && mx > 0.0 && std::isfinite(mx)) ? mx / 32767.0 : 1.0;
-            // the kernels dequantise with the FP32 scale: quantise with the same value
-            keep[c] = (float)sc[c];
-            sc[c] = (double)keep[c];
-        }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(comp_scale, sc, sizeof(sc), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    }
-    if (e == cudaSuccess)
-        e = launch_pack_links(g->g, canon, prec, recon, hop, g->r12_inv_scale, *out, err_bits,
-                              prec == HISQ_F16 ? comp_scale : nullptr, s);
-    unsigned long long bits = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, err_bits, sizeof(bits), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(scratch);
-    HISQ_CUDA(e);
-    double err;
-    memcpy(&err, &bits, sizeof(err));
-    if (!(err <= recon_tol))
-        return fail(HISQ_ERECON, "%s links are not representable with %d reals: max reconstruct error %.3e > tol %.3e",
-                    name, recon, err, recon_tol);
-    return HISQ_OK;
-}
-
-// Whether the FP64 links go into fixed point, and their block exponents: in
-// every (field, direction) all links finite and every nonzero link's largest
+// Checks both fields against recon_tol, sets the 16-bit component scales and
+// decides the FP64 format from what the scan found. Fixed point needs, in
+// every (field, direction), all links finite and every nonzero link's largest
 // real within a factor of 16 of the block's largest, so that the smallest
 // links still carry 51 bits (Haar links x a constant lie within 2.5).
-hisq_status choose_fx(hisq_gauge g, const double2* cu, const double2* cn, cudaStream_t s) {
-    unsigned long long* range = nullptr;
-    HISQ_CUDA(cudaMalloc(&range, 16 * sizeof(unsigned long long)));
-    unsigned long long bits[16] = {0};
-    cudaError_t e = launch_link_range(g->g, cu, range, s);
-    if (e == cudaSuccess) e = launch_link_range(g->g, cn, range + 8, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(bits, range, sizeof(bits), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(range);
-    HISQ_CUDA(e);
+hisq_status plan_links(hisq_gauge g, const LinkScan (&scan)[2], double recon_tol, LinkScales (&sc)[2]) {
+    auto real = [](unsigned long long b) {
+        double v;
+        memcpy(&v, &b, sizeof(v));
+        return v;
+    };
     g->fx = 1;
-    for (int f = 0; f < 2; ++f)
+    for (int f = 0; f < 2; ++f) {
+        const int recon = f ? g->recon_N : g->recon_U;
+        const double err = real(scan[f].err);
+        if (!(err <= recon_tol))
+            return fail(HISQ_ERECON, "%s links are not representable with %d reals: max reconstruct error %.3e > tol %.3e",
+                        f ? "Naik" : "fat", recon, err, recon_tol);
+        float* keep = f ? g->lscale_n : g->lscale_u;
+        for (int c = 0; c < 9; ++c) {
+            const double mx = real(scan[f].comp[c]);
+            const bool used = g->prec == HISQ_F16 && c < recon / 2 && mx > 0.0 && std::isfinite(mx);
+            // the kernels dequantise with the FP32 scale: quantise with the same value
+            keep[c] = used ? (float)(mx / 32767.0) : 1.0f;
+            sc[f].inv[c] = keep[c] > 0.0f ? 1.0 / (double)keep[c] : 0.0;
+        }
         for (int mu = 0; mu < 4; ++mu) {
-            double hi, lo;
-            memcpy(&hi, &bits[8 * f + mu], sizeof(hi));
-            memcpy(&lo, &bits[8 * f + 4 + mu], sizeof(lo));
+            const double hi = real(scan[f].hi[mu]), lo = real(~scan[f].nlo[mu]);
             int ex = 0;
             if (hi > 0.0 && std::isfinite(hi)) std::frexp(hi, &ex);
             g->fx_exp[4 * f + mu] = ex;
+            sc[f].fx_exp[mu] = ex;
             if (!std::isfinite(hi) || (hi > 0.0 && !(lo >= hi / 16.0)) || ex < -200 || ex > 200) g->fx = 0;
         }
+    }
     return HISQ_OK;
 }
 
-hisq_status pack_field_fx(hisq_gauge g, const double2* canon, int field, double2** out, size_t* bytes,
-                          cudaStream_t s) {
-    const size_t sz = 2 * 4 * 9 * (size_t)g->g.vh * sizeof(double2);
-    HISQ_CUDA(cudaMalloc(out, sz));
-    *bytes += sz;
-    double sc[4];
-    for (int mu = 0; mu < 4; ++mu) sc[mu] = std::ldexp(1.0, 55 - g->fx_exp[4 * field + mu]);
-    double* scale = nullptr;
-    HISQ_CUDA(cudaMalloc(&scale, sizeof(sc)));
-    cudaError_t e = cudaMemcpyAsync(scale, sc, sizeof(sc), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_pack_links_fx(g->g, canon, scale, *out, s);
+// Scans both canonical fields, then packs each in one pass (its FP64 copy and
+// its storage copy) into one allocation: a cudaFree costs about 0.3 ms
+// whatever its size, a cudaMalloc 0.3 us per MB.
+hisq_status pack_links(hisq_gauge g, const double2* cu, const double2* cn, double recon_tol, cudaStream_t s) {
+    const double2* canon[2] = {cu, cn};
+    const int recon[2] = {g->recon_U, g->recon_N};
+    LinkScan* scan_d = nullptr;
+    LinkScan scan[2];
+    LinkScales sc[2];
+    HISQ_CUDA(cudaMalloc(&scan_d, sizeof(scan)));
+    cudaError_t e = cudaSuccess;
+    for (int f = 0; f < 2 && e == cudaSuccess; ++f)
+        e = launch_link_scan(g->g, canon[f], recon[f], f ? 3 : 1, g->r12_inv_scale, scan_d + f, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scan, scan_d, sizeof(scan), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(scale);
+    cudaFree(scan_d);
     HISQ_CUDA(e);
+    hisq_status st = plan_links(g, scan, recon_tol, sc);
+    if (st != HISQ_OK) return st;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    size_t off[5] = {0, 0, 0, 0, 0};   // U64, N64, U_lo, N_lo
+    for (int i = 0; i < 4; ++i) {
+        const size_t nc = i < 2 ? 9 : recon[i - 2] / 2;
+        size_t sz = 2 * 4 * nc * (size_t)g->g.vh * prec_complex_bytes(i < 2 ? HISQ_F64 : g->prec);
+        if (i >= 2 && g->prec == HISQ_F64) sz = 0;
+        g->link_bytes += sz;
+        off[i + 1] = off[i] + up(sz);
+    }
+    HISQ_CUDA(cudaMalloc(&g->link_block, off[4]));
+    char* base = (char*)g->link_block;
+    g->U64 = (double2*)base;
+    g->N64 = (double2*)(base + off[1]);
+    g->U_lo = g->prec == HISQ_F64 ? (void*)g->U64 : base + off[2];
+    g->N_lo = g->prec == HISQ_F64 ? (void*)g->N64 : base + off[3];
+    HISQ_CUDA(launch_pack_links(g->g, cu, g->prec, g->recon_U, g->fx, sc[0], g->U64, g->U_lo, s));
+    HISQ_CUDA(launch_pack_links(g->g, cn, g->prec, g->recon_N, g->fx, sc[1], g->N64, g->N_lo, s));
+    HISQ_CUDA(cudaStreamSynchronize(s));
     return HISQ_OK;
 }
 
 void destroy_gauge(hisq_gauge g) {
     if (!g) return;
     for (Workspace* w : g->ws) free_workspace(w);
-    if (g->U_lo && g->U_lo != g->U64) cudaFree(g->U_lo);
-    if (g->N_lo && g->N_lo != g->N64) cudaFree(g->N_lo);
-    if (g->U64) cudaFree(g->U64);
-    if (g->N64) cudaFree(g->N64);
+    if (g->link_block) cudaFree(g->link_block);
     if (g->mdagm_tmp) cudaFree(g->mdagm_tmp);
     if (g->dot_partials) cudaFree(g->dot_partials);
     if (g->dot_counter) cudaFree(g->dot_counter);
@@ -379,26 +361,8 @@ extern "C" hisq_status hisq_gauge_load(const int L[4], const void* U, const void
         if (!(sc > 0.0)) return cleanup(fail(HISQ_ERECON, "R12 needs a nonzero first row in U[0][0]"));
         g->r12_inv_scale = 1.0 / sc;
     }
-    size_t bytes = 0;
-    st = choose_fx(g, cu, cn, s);
-    if (st == HISQ_OK && g->fx) {
-        st = pack_field_fx(g, cu, 0, &g->U64, &bytes, s);
-        if (st == HISQ_OK) st = pack_field_fx(g, cn, 1, &g->N64, &bytes, s);
-    } else if (st == HISQ_OK) {
-        st = pack_field(g, cu, HISQ_F64, 18, 1, recon_tol, (void**)&g->U64, &bytes, "fat", s);
-        if (st == HISQ_OK) st = pack_field(g, cn, HISQ_F64, 18, 3, recon_tol, (void**)&g->N64, &bytes, "Naik", s);
-    }
-    if (st == HISQ_OK) {
-        if (prec == HISQ_F64) {
-            g->U_lo = g->U64;
-            g->N_lo = g->N64;
-        } else {
-            st = pack_field(g, cu, prec, recon_U, 1, recon_tol, &g->U_lo, &bytes, "fat", s);
-            if (st == HISQ_OK) st = pack_field(g, cn, prec, recon_N, 3, recon_tol, &g->N_lo, &bytes, "Naik", s);
-        }
-    }
+    st = pack_links(g, cu, cn, recon_tol, s);
     if (st != HISQ_OK) return cleanup(st);
-    g->link_bytes = bytes;
     *out = g;
     return cleanup(HISQ_OK);
 }

@@ -297,28 +297,27 @@ cudaError_t launch_transpose_spinor(const double2* in, double2* out, int n, int 
 // ---------------------------------------------------------------------------
 // Link packing (gauge.cu)
 // ---------------------------------------------------------------------------
-// Pack canonical complex128 [4][V][3][3] into [2][4][ncomp][vh] of `prec`,
-// with reconstruct residual max written (as ordered bits) to *err_bits.
-// F16 links are 16-bit fixed point: comp_scale[c] (device, FP64) is the
-// scale of stored component c (see launch_link_absmax); ignored otherwise.
-cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon,
-                              int hop, double r12_inv_scale, void* out,
-                              unsigned long long* err_bits, const double* comp_scale,
-                              cudaStream_t s);
-// Largest |Re| or |Im| of every stored component (recon / 2 of them) over the
-// field, as the bits of non-negative doubles OR-maximised into maxbits[c].
-cudaError_t launch_link_absmax(const Geom& g, const double2* canon, int recon, int hop,
-                               double r12_inv_scale, unsigned long long* maxbits, cudaStream_t s);
-// Range of the links of a field, per direction mu: the bits of the largest
-// |Re|, |Im| into range[mu] (+inf if any is not finite) and of the smallest
-// over nonzero links of a link's largest into range[4 + mu] (+inf if none).
-// range: 8 device values, set by the call.
-cudaError_t launch_link_range(const Geom& g, const double2* canon, unsigned long long* range, cudaStream_t s);
-// Pack canonical links into the fixed-point FP64 storage (dslash_fx64.cuh):
-// R18 components as int4 limbs (re1, re0, im1, im0) of value * scale[mu],
-// scale (device) = 2^(55 - e) of each direction.
-cudaError_t launch_pack_links_fx(const Geom& g, const double2* canon, const double* scale, void* out,
-                                 cudaStream_t s);
+// What one pass over a canonical field finds (all values are the bits of
+// non-negative doubles): the largest |Re|, |Im| of every stored component
+// (recon / 2 of them), per direction the largest over all reals and the
+// complement of the smallest over nonzero links of a link's largest (0 if
+// there is none), and the largest reconstruct error.
+struct LinkScan {
+    unsigned long long comp[9], hi[4], nlo[4], err;
+};
+cudaError_t launch_link_scan(const Geom& g, const double2* canon, int recon, int hop, double r12_inv_scale,
+                             LinkScan* out, cudaStream_t s);
+// Pack canonical complex128 [4][V][3][3] into the FP64 copy out64 [2][4][9][vh]
+// (doubles, or with fx int4 limbs (re1, re0, im1, im0) of value 2^(55 - sc.fx_exp[mu]),
+// see dslash_fx64.cuh) and, for F32 / F16, into the storage copy out_lo
+// [2][4][recon / 2][vh]. F16 links are 16-bit fixed point, value * sc.inv[c]
+// rounded for stored component c.
+struct LinkScales {
+    int fx_exp[4];
+    double inv[9];
+};
+cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, int fx, const LinkScales& sc,
+                              void* out64, void* out_lo, cudaStream_t s);
 // Compress to double [4][V][r] and back (ABI helpers).
 cudaError_t launch_compress_links(const Geom& g, const double2* canon, int recon, int hop,
                                   double r12_inv_scale, double* packed,
