@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(kThreads) update_r_kernel(BlasArgs a, void* r,
     }
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[1] = {false};
-    if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals)) finish_cg_beta(a.cg, s_vals, a.n);
+    if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
+        finish_cg_beta(a.cg, threadIdx.x, s_vals[threadIdx.x]);
 }
 
 // x += alpha p ; p = r + beta p, both from the old p, in one pass. alpha is
@@ -306,8 +307,8 @@ __global__ void __launch_bounds__(kThreads) copy_residual_kernel(BlasArgs a, con
     }
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[2] = {false, true};
-    if (block_reduce_arrive<double, 2>(a.red, val, a.n, mx, s_vals))
-        finish_reliable(a.cg, s_vals, a.n, tol2);
+    if (block_reduce_arrive<double, 2>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
+        finish_reliable(a.cg, threadIdx.x, s_vals[2 * threadIdx.x], s_vals[2 * threadIdx.x + 1], tol2);
 }
 
 // r_lo = scale r_hi ; p_lo = reset ? r_lo : p_lo * scale/scale_old ; rr = |r_lo|^2
@@ -392,7 +393,8 @@ __global__ void __launch_bounds__(kThreads) dot_alpha_kernel(BlasArgs a, const v
     }
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[1] = {false};
-    if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals)) finish_cg_alpha(a.cg, s_vals, a.n);
+    if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
+        finish_cg_alpha(a.cg, threadIdx.x, s_vals[threadIdx.x]);
 }
 
 // |r_hi|^2 and max |r_i| -> reliable finish (full-lattice residual)
@@ -410,8 +412,38 @@ __global__ void __launch_bounds__(kThreads) residual_norm_kernel(BlasArgs a, con
     }
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[2] = {false, true};
-    if (block_reduce_arrive<double, 2>(a.red, val, a.n, mx, s_vals))
-        finish_reliable(a.cg, s_vals, a.n, tol2);
+    if (block_reduce_arrive<double, 2>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
+        finish_reliable(a.cg, threadIdx.x, s_vals[2 * threadIdx.x], s_vals[2 * threadIdx.x + 1], tol2);
+}
+
+// Sums of a reduction over its nslots blocks, one block per rhs, and the finish.
+__global__ void __launch_bounds__(kThreads) red_finish_kernel(RedScratch red, int nslots, int nv, int finish,
+                                                              CgScalars* cg, double* out, double tol2) {
+    const int k = blockIdx.x;
+    __shared__ double s_w[2][kThreads / 32];
+    for (int j = 0; j < nv; ++j) {
+        const double* src = red.partials + (size_t)(k * nv + j) * kMaxRedBlocks;
+        constexpr int U = 4;
+        double acc = 0.0;
+        for (int i0 = threadIdx.x; i0 < nslots; i0 += U * kThreads) {
+            double t[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) t[u] = i0 + u * kThreads < nslots ? __ldcg(src + i0 + u * kThreads) : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc = j ? fmax(acc, t[u]) : acc + t[u];
+        }
+        acc = j ? warp_max(acc) : warp_sum(acc);
+        if ((threadIdx.x & 31) == 0) s_w[j][threadIdx.x >> 5] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v0 = 0.0, v1 = 0.0;
+        for (int w = 0; w < kThreads / 32; ++w) {
+            v0 += s_w[0][w];
+            if (nv == 2) v1 = fmax(v1, s_w[1][w]);
+        }
+        finish_rhs(finish, cg, out, k, nv, v0, v1, tol2);
+    }
 }
 
 // [h][V_h][3] <-> [h][3][V_h] per rhs (FP64 complex)
@@ -486,6 +518,12 @@ cudaError_t launch_dot_alpha(const BlasArgs& a, int prec, const void* p, const v
                              cudaStream_t s) {
     HISQ_PREC_SWITCH(prec, (dot_alpha_kernel<S><<<blas_grid(a.len / vec_n<S>(), a.n), kThreads, 0, s>>>(
                                 a, p, Ap)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_red_finish(const DslashArgs& a, int nslots, cudaStream_t s) {
+    const int nv = a.red_mode == RED_NORM_MAX_W ? 2 : 1;
+    red_finish_kernel<<<a.nrhs, kThreads, 0, s>>>(a.red, nslots, nv, a.finish, a.cg, a.red_out, a.tol2);
     return cudaGetLastError();
 }
 

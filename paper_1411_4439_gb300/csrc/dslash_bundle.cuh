@@ -30,8 +30,9 @@
 //                             the code: no instruction-fetch stalls);
 //   BundleHopsStaged          unrolled, the neighbour chunks copied into
 //                             shared memory D hops ahead by per-thread cp.async;
-//   BundleHopsCompactStaged   the compact loop with that staging (D = 1 or 3),
-//                             the default for FP16 storage.
+//   BundleHopsCompactStaged   the compact loop with that staging (D = 1 or 3)
+//                             of the neighbour chunks and of the links, the
+//                             default for FP16 storage.
 // Sites are visited plane by plane with the longer of z and t slow
 // (visit_site), so the neighbour chunks stay in L2 between their readers.
 #pragma once
@@ -100,6 +101,29 @@ __device__ __forceinline__ float2 stored_rhs(float2 v, __half) {
 // Asynchronous 16-byte copies global -> shared (L1 bypassed).
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// The same through L1, 4, 8 or 16 bytes.
+template <int BYTES>
+__device__ __forceinline__ void cp_async_ca(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
+}
+// One pair / one single link component from shared memory.
+__device__ __forceinline__ void ld_shared(uint32_t ad, short2& a, short2& b) {
+    uint2 w;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w.x), "=r"(w.y) : "r"(ad));
+    memcpy(&a, &w.x, 4);
+    memcpy(&b, &w.y, 4);
+}
+__device__ __forceinline__ void ld_shared(uint32_t ad, short2& a) {
+    unsigned w;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(ad));
+    memcpy(&a, &w, 4);
+}
+__device__ __forceinline__ void ld_shared(uint32_t ad, float2& a, float2& b) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y) : "r"(ad));
+}
+__device__ __forceinline__ void ld_shared(uint32_t ad, float2& a) {
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a.x), "=f"(a.y) : "r"(ad));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -670,13 +694,26 @@ struct BundleHopsStaged {
 };
 
 // Compact hop loop (direction as a runtime loop, a quarter of the code, so
-// the warps of an SM share a small instruction footprint) with the
-// neighbour chunks staged in shared memory D hops ahead as in
-// BundleHopsStaged; D = 1 or 3, so the stage of hop 4 mu + HOP is fixed by
-// HOP alone (NS = D + 1 divides 4).
-template <typename S, typename LS, int RU, int RN, int R, int D>
+// the warps of an SM share a small instruction footprint) with the neighbour
+// chunks and the links staged in shared memory D hops ahead by per-thread
+// cp.async; D = 1 or 3, so the stage of hop 4 mu + HOP is fixed by HOP alone
+// (NS = D + 1 divides 4). T is the block's thread count, ONE whether the block
+// has one rhs group: chunk and link addresses are then uniform bases plus one
+// 32-bit thread offset. Per stage the block holds 3 NG planes of T chunks and
+// the link's component pairs as NCMAX / 2 planes of T words (8 bytes for
+// 16-bit links, 16 for FP32) plus one plane of T single components.
+//
+// 48^3x12, n = 8, FP16 (EPI_NONE / EPI_X): 203 / 208 us with the next link in
+// registers (its load was a quarter of the stalls), 188 / 201 with the links
+// staged, 186 / 193 with uniform addresses, 170 / 175 with a block per tile.
+// What bounds it now: the FMA pipe. A packed FMA with fresh operands takes 2.7
+// cycles of a scheduler (register ports), so the 144 of a hop take 390 of the
+// 645 cycles of a warp's hop. FP32 storage stays on BundleHops: twice the
+// bytes through shared memory make this loop 228 us against 202.
+template <typename S, typename LS, int RU, int RN, int R, int D, int T, bool ONE>
 struct BundleHopsCompactStaged {
     using LC = typename Traits<LS>::C;
+    using LV = typename LinkPair<LC>::V;
     static constexpr int W = Bundle<S>::W;
     static constexpr int NG = R / W;
     static constexpr int P = R / 2;
@@ -684,29 +721,31 @@ struct BundleHopsCompactStaged {
     static constexpr int NCN = (RN == 18) ? 9 : (RN == 14 ? 7 : 6);
     static constexpr int NCMAX = NCU > NCN ? NCU : NCN;
     static constexpr int NS = D + 1;
+    static constexpr uint32_t kChunkStage = 3u * NG * 16u * T;
+    static constexpr uint32_t kLinkStage = NCMAX * (uint32_t)sizeof(LC) * T;
+    // the single component's plane, after the pairs of the larger link: a stage
+    // serves fat and Naik hops, and no thread may touch another's words
+    static constexpr uint32_t kSingle = (NCMAX / 2) * (uint32_t)sizeof(LV) * T;
+    static constexpr uint32_t kBytes = NS * (kChunkStage + kLinkStage);
     static_assert(4 % NS == 0, "the stage of a hop must not depend on its direction");
-
-    struct Lk {
-        LC l[NCMAX];
-    };
 
     const DslashArgs& a;
     const LC* __restrict__ Ub;
     const LC* __restrict__ Nb;
-    const uint4* __restrict__ in;
-    uint32_t slot0;
-    uint32_t tstride;
+    const char* in;
+    uint32_t base;   // shared address of the block's stages
+    uint32_t tid;
     int vh, p, q, h, hrow, x, y, z, t;
     f2x (&ar)[P][3];
     f2x (&ai)[P][3];
 
-    __device__ __forceinline__ BundleHopsCompactStaged(const DslashArgs& args, int h_, int k0, uint32_t slot0_,
-                                                       uint32_t tstride_, f2x (&ar_)[P][3], f2x (&ai_)[P][3])
-        : a(args), slot0(slot0_), tstride(tstride_), ar(ar_), ai(ai_) {
+    __device__ __forceinline__ BundleHopsCompactStaged(const DslashArgs& args, int h_, int k0, uint32_t base_, int tid_,
+                                                       f2x (&ar_)[P][3], f2x (&ai_)[P][3])
+        : a(args), base(base_), tid(tid_), ar(ar_), ai(ai_) {
         Ub = reinterpret_cast<const LC*>(a.U);
         Nb = reinterpret_cast<const LC*>(a.N);
         vh = a.g.vh;
-        in = reinterpret_cast<const uint4*>(a.in[0]) + (size_t)(k0 / W) * 3 * vh;
+        in = reinterpret_cast<const char*>(a.in[0]) + (ONE ? 0 : (size_t)(k0 / W) * 3 * vh * 16);
         p = a.parity;
         q = 1 - p;
         h = h_;
@@ -732,43 +771,67 @@ struct BundleHopsCompactStaged {
         return h + (cn - c) * stride;
     }
 
+    // shared address of the pairs / the single component of hop HOP's link
     template <int HOP>
-    __device__ __forceinline__ void issue_link(int mu, Lk& b) const {
+    __device__ __forceinline__ uint32_t link_slot() const {
+        return base + NS * kChunkStage + (HOP % NS) * kLinkStage;
+    }
+
+    // asynchronous copies of hop HOP of direction mu into its stage, one group
+    template <int HOP>
+    __device__ __forceinline__ void stage(int mu) const {
         constexpr bool NAIK = HOP >= 2;
         constexpr bool BACK = HOP & 1;
         constexpr int NC = NAIK ? NCN : NCU;
-        const LC* base = (NAIK ? Nb : Ub) + (size_t)((BACK ? q : p) * 4 + mu) * NC * vh;
-        const int li = BACK ? neighbour<HOP>(mu) : h;
-        load_link_raw<LC, NC>(b.l, base, vh, li);
-    }
-
-    template <int HOP>
-    __device__ __forceinline__ void stage(int mu) const {
         const int hn = neighbour<HOP>(mu);
-        const uint32_t st = slot0 + (uint32_t)((HOP % NS) * 3 * NG) * tstride;
+        const uint32_t st = base + (HOP % NS) * kChunkStage + 16u * tid;
+        const size_t plane = (size_t)vh * 16;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
             for (int g = 0; g < NG; ++g)
-                cp_async16(st + (uint32_t)(c * NG + g) * tstride, in + (size_t)(g * 3 + c) * vh + hn);
+                cp_async16(st + (uint32_t)(c * NG + g) * 16u * T, in + (g * 3 + c) * plane + (uint32_t)hn * 16u);
+        const LC* block = (NAIK ? Nb : Ub) + (size_t)((BACK ? q : p) * 4 + mu) * NC * vh;
+        const uint32_t li = (uint32_t)(BACK ? hn : h);
+        const char* pb = reinterpret_cast<const char*>(block);
+        const uint32_t sl = link_slot<HOP>();
+#pragma unroll
+        for (int pp = 0; pp < NC / 2; ++pp)
+            cp_async_ca<sizeof(LV)>(sl + (pp * T + tid) * (uint32_t)sizeof(LV),
+                                    pb + (size_t)pp * vh * sizeof(LV) + li * (uint32_t)sizeof(LV));
+        if constexpr (NC & 1)
+            cp_async_ca<sizeof(LC)>(sl + kSingle + tid * (uint32_t)sizeof(LC),
+                                    pb + (size_t)(NC / 2) * vh * sizeof(LV) + li * (uint32_t)sizeof(LC));
         cp_async_commit();
     }
 
     template <int HOP>
-    __device__ __forceinline__ void compute(int mu, const Lk& b) {
+    __device__ __forceinline__ void fetch_link(LC (&l)[NCMAX]) const {
+        constexpr int NC = HOP >= 2 ? NCN : NCU;
+        const uint32_t sl = link_slot<HOP>();
+#pragma unroll
+        for (int pp = 0; pp < NC / 2; ++pp)
+            ld_shared(sl + (pp * T + tid) * (uint32_t)sizeof(LV), l[2 * pp], l[2 * pp + 1]);
+        if constexpr (NC & 1) ld_shared(sl + kSingle + tid * (uint32_t)sizeof(LC), l[NC - 1]);
+    }
+
+    template <int HOP>
+    __device__ __forceinline__ void compute(int mu) {
         constexpr bool NAIK = HOP >= 2;
         constexpr bool BACK = HOP & 1;
         constexpr int REC = NAIK ? RN : RU;
         constexpr int NC = NAIK ? NCN : NCU;
+        LC l[NCMAX];
+        fetch_link<HOP>(l);
         const float* sc = NAIK ? a.lscale_n : a.lscale_u;
         Link<float2> m;
 #pragma unroll
-        for (int c = 0; c < 6; ++c) m.e[c] = link_elem(b.l[c], sc[c]);
+        for (int c = 0; c < 6; ++c) m.e[c] = link_elem(l[c], sc[c]);
         if constexpr (REC == 18) {
 #pragma unroll
-            for (int c = 6; c < 9; ++c) m.e[c] = link_elem(b.l[c], sc[c]);
+            for (int c = 6; c < 9; ++c) m.e[c] = link_elem(l[c], sc[c]);
         } else if constexpr (REC == 14) {
-            third_row(m, link_elem(b.l[NC - 1], sc[NC - 1]));
+            third_row(m, link_elem(l[NC - 1], sc[NC - 1]));
         } else {
             const int e = mu == 0 ? 0 : mu == 1 ? x : mu == 2 ? (x + y) : (x + y + z);
             int sgn = (e & 1) ? -1 : 1;
@@ -780,13 +843,13 @@ struct BundleHopsCompactStaged {
             const double f = HOP == 0 ? a.ft1 : HOP == 1 ? a.bt1 : HOP == 2 ? a.ft3 : a.bt3;
             scale_link(m, (float)f);
         }
-        const uint32_t st = slot0 + (uint32_t)((HOP % NS) * 3 * NG) * tstride;
+        const uint32_t st = base + (HOP % NS) * kChunkStage + 16u * tid;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             uint4 ch[NG];
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
-                const uint32_t ad = st + (uint32_t)(j * NG + g) * tstride;
+                const uint32_t ad = st + (uint32_t)(j * NG + g) * 16u * T;
                 asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                              : "=r"(ch[g].x), "=r"(ch[g].y), "=r"(ch[g].z), "=r"(ch[g].w)
                              : "r"(ad));
@@ -812,17 +875,13 @@ struct BundleHopsCompactStaged {
         }
     }
 
-    // stage hop e + D (direction mu + (HOP + D) / 4), load the next link,
-    // wait for hop e's chunks, multiply
+    // stage hop e + D (direction mu + (HOP + D) / 4), wait for hop e's copies,
+    // multiply
     template <int HOP>
-    __device__ __forceinline__ void step(int mu, Lk (&lk)[2]) {
+    __device__ __forceinline__ void step(int mu) {
         constexpr int SH = (HOP + D) & 3;                 // hop index of e + D within its direction
         const int smu = mu + (HOP + D) / 4;               // its direction
-        const bool staged_more = smu < 4;
-        if (staged_more) stage<SH>(smu);
-        constexpr int NEXT = (HOP + 1) & 3;
-        const int nmu = HOP == 3 ? mu + 1 : mu;
-        if (nmu < 4) issue_link<NEXT>(nmu, lk[NEXT & 1]);
+        if (smu < 4) stage<SH>(smu);
         // groups committed after hop e's: D while later hops were staged, fewer at the end
         const int remaining = 15 - (4 * mu + HOP);
         if (remaining >= D)
@@ -833,22 +892,20 @@ struct BundleHopsCompactStaged {
             cp_async_wait<(D >= 2 ? 1 : 0)>();
         else
             cp_async_wait<0>();
-        compute<HOP>(mu, lk[HOP & 1]);
+        compute<HOP>(mu);
     }
 
     __device__ __forceinline__ void run() {
-        Lk lk[2];
-        issue_link<0>(0, lk[0]);
         // prologue: hops 0 .. D-1 of direction 0
         stage<0>(0);
         if constexpr (D >= 2) stage<1>(0);
         if constexpr (D >= 3) stage<2>(0);
 #pragma unroll 1
         for (int mu = 0; mu < 4; ++mu) {
-            step<0>(mu, lk);
-            step<1>(mu, lk);
-            step<2>(mu, lk);
-            step<3>(mu, lk);
+            step<0>(mu);
+            step<1>(mu);
+            step<2>(mu);
+            step<3>(mu);
         }
     }
 };
@@ -857,24 +914,22 @@ struct BundleHopsCompactStaged {
 // or out = cx x + cd (D in) with optionally Re<x, out> per rhs (EPI_X), for
 // the rhs of every thread group. a.in[0], a.out[0], a.x[0] are bundle bases.
 template <typename S, typename LS, int RU, int RN, int R, int MINB, bool PK, int LD, int SD, int EPI,
-          bool COMPACT, int STAGE = 0>
+          bool COMPACT, int STAGE = 0, bool ONE = false>
 __global__ void __launch_bounds__(128, MINB) dslash_bundle_kernel(const DslashArgs a) {
     constexpr int W = Bundle<S>::W;
     constexpr int NG = R / W;
     constexpr int P = R / 2;
     const int vh = a.g.vh;
-    const int k0 = threadIdx.y * R;
+    const int k0 = ONE ? 0 : threadIdx.y * R;   // ONE: the launcher checked nrhs == R
     const size_t gofs = (size_t)(k0 / W) * 3 * vh;
 
-    float red0[R], red1[R];
+    __shared__ RedParts parts;
+    const int vb = blockIdx.x * a.run * blockDim.x;
+    for (int it = 0, v = vb + threadIdx.x; it < a.run && v - (int)threadIdx.x < vh; ++it, v += blockDim.x) {
+        float red0[R];
 #pragma unroll
-    for (int j = 0; j < R; ++j) {
-        red0[j] = 0.f;
-        red1[j] = 0.f;
-    }
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v - (int)threadIdx.x < vh;
-         v += gridDim.x * blockDim.x) {
-        if (v >= vh) continue;
+        for (int j = 0; j < R; ++j) red0[j] = 0.f;
+        if (v < vh) {
         const int h = visit_site(v, a.g);
         if constexpr (EPI == EPI_X) {
             // the epilogue's x is read after the hops; start it towards L2 now
@@ -931,8 +986,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_bundle_kernel(const DslashAr
             extern __shared__ __align__(16) unsigned char bundle_smem[];
             const int tid = threadIdx.x + threadIdx.y * blockDim.x;
             const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(bundle_smem));
-            BundleHopsCompactStaged<S, LS, RU, RN, R, STAGE - 10> hops(a, h, k0, base + 16u * tid,
-                                                                       16u * blockDim.x * blockDim.y, ar, ai);
+            BundleHopsCompactStaged<S, LS, RU, RN, R, STAGE - 10, 128, ONE> hops(a, h, k0, base, tid, ar, ai);
             hops.run();
         } else if constexpr (STAGE > 0 && STAGE < 10) {
             extern __shared__ __align__(16) unsigned char bundle_smem[];
@@ -986,9 +1040,12 @@ __global__ void __launch_bounds__(128, MINB) dslash_bundle_kernel(const DslashAr
                 }
                 ob[(size_t)(g * 3 + c) * vh] = make_chunk(w, S{});
             }
+        }
+        // Re<x, out> is the only reduction of this kernel
+        if (EPI == EPI_X && a.red_mode != RED_NONE) tile_reduce<R>(a, k0, red0, red0, parts, it == 0);
     }
     if (a.red_mode == RED_NONE) return;
-    block_reduce_finish<R>(a, k0, red0, red1);
+    block_finish(a, parts);
 }
 
 // Whether (n, rhs per thread) fits the bundle kernel of storage S.
@@ -998,16 +1055,19 @@ __host__ __device__ constexpr bool bundle_shape_ok(int n, int rpt) {
 }
 
 template <typename S, typename LS, int RU, int RN, int R, int MINB, bool PK, int LD, int SD, int EPI,
-          bool COMPACT, int STAGE = 0>
-cudaError_t launch_dslash_bundle(const DslashArgs& a, cudaStream_t s) {
+          bool COMPACT, int STAGE = 0, bool ONE = false>
+cudaError_t launch_dslash_bundle(const DslashArgs& args, cudaStream_t s) {
+    DslashArgs a = args;
     if (a.t_only || !bundle_shape_ok<S>(a.nrhs, R)) return cudaErrorInvalidValue;
     if (EPI == EPI_NONE && a.red_mode != RED_NONE) return cudaErrorInvalidValue;
     const int G = a.nrhs / R;
     if (G > 4) return cudaErrorInvalidValue;
-    const int bx = 128 / G;   // 128 threads: 128 / G sites x G rhs groups
+    if constexpr (STAGE > 10 && STAGE < 30 && !ONE) {
+        if (G == 1) return launch_dslash_bundle<S, LS, RU, RN, R, MINB, PK, LD, SD, EPI, COMPACT, STAGE, true>(a, s);
+    }
+    const int bx = (128 / G) & ~31;   // whole warps of sites x G rhs groups
     const dim3 block(bx, G);
-    auto* kern = dslash_bundle_kernel<S, LS, RU, RN, R, MINB, PK, LD, SD, EPI, COMPACT, STAGE>;
-    int occ = 0;
+    auto* kern = dslash_bundle_kernel<S, LS, RU, RN, R, MINB, PK, LD, SD, EPI, COMPACT, STAGE, ONE>;
     cudaError_t e = cudaSuccess;
     size_t smem = 0;
     if constexpr (STAGE == 30) {
@@ -1016,26 +1076,24 @@ cudaError_t launch_dslash_bundle(const DslashArgs& a, cudaStream_t s) {
         smem = (size_t)3 * (R / Bundle<S>::W) * xy_tile_rows(a.g.hx) * a.g.hx * 16;
         if (G != 1 || a.g.sz % 128 != 0 || smem > 100 * 1024)
             return launch_dslash_bundle<S, LS, RU, RN, R, MINB, PK, LD, SD, EPI, COMPACT, 0>(a, s);
-        // the tile's size follows the lattice: occupancy per call
+        // the tile's size follows the lattice
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, bx * G, smem);
         if (e != cudaSuccess) return e;
-        if (occ < 1) return cudaErrorInvalidConfiguration;
     } else {
-        // staged: (D + 1) stages x 3 R / W chunks of 16 bytes per thread, D = STAGE
-        // (unrolled loop) or STAGE - 10 (compact loop)
-        constexpr int DEPTH = STAGE > 10 ? STAGE - 10 : STAGE;
-        smem = DEPTH > 0 ? (size_t)(DEPTH + 1) * 3 * (R / Bundle<S>::W) * 16 * 128 : 0;
-        static OccCache cache;   // this kernel instance's occupancy per device
+        // staged chunks: (D + 1) stages x 3 R / W chunks of 16 bytes per thread, D = STAGE
+        // (unrolled loop); D = STAGE - 10 with the links too (compact loop)
+        if constexpr (STAGE > 10)
+            smem = BundleHopsCompactStaged<S, LS, RU, RN, R, STAGE - 10, 128, ONE>::kBytes;
+        else
+            smem = STAGE > 0 ? (size_t)(STAGE + 1) * 3 * (R / Bundle<S>::W) * 16 * 128 : 0;
+        static OccCache cache;   // sets this kernel instance's shared-memory attributes once per device
+        int occ = 0;
         e = cached_occupancy(cache, kern, bx * G, smem, G, &occ);
         if (e != cudaSuccess) return e;
     }
-    long long nblk = ((long long)a.g.vh + bx - 1) / bx;
-    const long long cap = (long long)occ * device_sm_count();
-    if (nblk > cap) nblk = cap;
-    if (nblk > kMaxRedBlocks) nblk = kMaxRedBlocks;
-    kern<<<(unsigned)nblk, block, smem, s>>>(a);
-    return cudaGetLastError();
+    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + bx - 1) / bx);
+    kern<<<blocks, block, smem, s>>>(a);
+    return finish_launch(a, blocks, s);
 }
 
 }  // namespace hisq

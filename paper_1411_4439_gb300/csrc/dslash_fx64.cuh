@@ -361,7 +361,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dslash_fx64_kernel(const __grid_co
 #pragma unroll
     for (int j = 0; j < R; ++j) red0[j] = red1[j] = 0.0;
 
-    for (int v = blockIdx.x * spb + slot; v - slot < vh; v += gridDim.x * spb) {
+    const int v0 = blockIdx.x * a.run * spb;
+    for (int it = 0, v = v0 + slot; it < a.run && v - slot < vh; ++it, v += spb) {
         if (SPLIT == 1 && v >= vh) continue;
         const int h = visit_site(v < vh ? v : vh - 1, a.g);
         FxHops<R, LAYOUT> hops(a, h, k0);
@@ -455,12 +456,9 @@ cudaError_t launch_fx64(const DslashArgs& args, cudaStream_t s) {
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
     const int spb = bx / SPLIT;
-    long long nblk = ((long long)a.g.vh + spb - 1) / spb;
-    const long long cap = (long long)occ * device_sm_count();
-    if (nblk > cap) nblk = cap;
-    if (nblk > kMaxRedBlocks) nblk = kMaxRedBlocks;
-    kern<<<(unsigned)nblk, dim3(bx, G), 0, s>>>(a);
-    return cudaGetLastError();
+    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + spb - 1) / spb);
+    kern<<<blocks, dim3(bx, G), 0, s>>>(a);
+    return finish_launch(a, blocks, s);
 }
 
 }  // namespace hisq

@@ -486,45 +486,58 @@ __device__ __forceinline__ void epilogue_site(const DslashArgs& a, int h, int k0
     }
 }
 
-// Per-rhs block reduction (warp tree -> shared -> partial slot) and the
-// last-block finish. Called by every thread of the block.
+// Per-warp sums of the block's tiles, one slot per value and warp of a group.
+struct RedParts {
+    double v[kMaxRedVals][8];
+};
+
+// Adds the reduction terms of one tile over the warp to its slots (sets them
+// at the first tile). Called by every lane of the warp.
 template <int RPT, typename R>
-__device__ __forceinline__ void block_reduce_finish(const DslashArgs& a, int k0, R (&red0)[RPT],
-                                                    R (&red1)[RPT]) {
-    // per-rhs block reduction: warp (fixed tree) -> shared -> partial slot
-    __shared__ double s_part[kMaxRedVals][8];
-    __shared__ double s_vals[kMaxRedVals];
+__device__ __forceinline__ void tile_reduce(const DslashArgs& a, int k0, R (&red0)[RPT], R (&red1)[RPT], RedParts& parts,
+                                            bool first) {
     const int nv = (a.red_mode == RED_NORM_MAX_W) ? 2 : 1;
     const int lane = threadIdx.x & 31;
     const int wig = threadIdx.x >> 5;            // warp index within the group
-    const int wpg = blockDim.x >> 5;             // warps per group
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-        const double s0 = (double)warp_sum(red0[j]);
-        const double s1 = (double)warp_max(red1[j]);
-        if (lane == 0) {
-            s_part[(k0 + j) * nv][wig] = s0;
-            if (nv == 2) s_part[(k0 + j) * nv + 1][wig] = s1;
-        }
+    const int k = k0 + multi_index<RPT>(lane);
+    const bool lead = lane % (32 / RPT) == 0;
+    const double s0 = (double)warp_multi<RPT>(red0, [](R p, R q) { return p + q; });
+    if (lead) parts.v[k * nv][wig] = first ? s0 : parts.v[k * nv][wig] + s0;
+    if (nv == 2) {
+        const double s1 = (double)warp_multi<RPT>(red1, [](R p, R q) { return (R)fmax(p, q); });
+        if (lead) parts.v[k * nv + 1][wig] = first ? s1 : fmax(parts.v[k * nv + 1][wig], s1);
     }
+}
+
+// The block's sums into its partial slot. With a.red_defer the sums over the
+// blocks and the finish are left to launch_red_finish; else the last block
+// does them. Called by every thread of the block.
+__device__ __forceinline__ void block_finish(const DslashArgs& a, const RedParts& parts) {
+    __shared__ double s_vals[kMaxRedVals];
+    const int nv = (a.red_mode == RED_NORM_MAX_W) ? 2 : 1;
+    const int wpg = (blockDim.x + 31) >> 5;      // warps per group
     __syncthreads();
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nvals = a.nrhs * nv;
     if (tid < nvals) {
         const bool is_max = (nv == 2) && (tid & 1);
         double acc = 0.0;
-        for (int w = 0; w < wpg; ++w) acc = is_max ? fmax(acc, s_part[tid][w]) : acc + s_part[tid][w];
+        for (int w = 0; w < wpg; ++w) acc = is_max ? fmax(acc, parts.v[tid][w]) : acc + parts.v[tid][w];
         a.red.partials[(size_t)tid * kMaxRedBlocks + blockIdx.x] = acc;
     }
+    if (a.red_defer) return;
     if (!last_block_arrive(a.red.counter, gridDim.x)) return;
     finish_values(a.red, nvals, gridDim.x, [nv](int v) { return nv == 2 && (v & 1); }, s_vals);
-    if (a.finish == FIN_CG_ALPHA) {
-        finish_cg_alpha(a.cg, s_vals, a.nrhs);
-    } else if (a.finish == FIN_RELIABLE) {
-        finish_reliable(a.cg, s_vals, a.nrhs, a.tol2);
-    } else if (a.red_out != nullptr && tid < nvals) {
-        a.red_out[tid] = s_vals[tid];
-    }
+    if (tid < a.nrhs)
+        finish_rhs(a.finish, a.cg, a.red_out, tid, nv, s_vals[tid * nv], nv == 2 ? s_vals[tid * nv + 1] : 0.0, a.tol2);
+}
+
+template <int RPT, typename R>
+__device__ __forceinline__ void block_reduce_finish(const DslashArgs& a, int k0, R (&red0)[RPT],
+                                                    R (&red1)[RPT]) {
+    __shared__ RedParts parts;
+    tile_reduce<RPT>(a, k0, red0, red1, parts, true);
+    block_finish(a, parts);
 }
 
 // Resident blocks per SM of one kernel, cached per device: every launcher
@@ -582,11 +595,39 @@ cudaError_t cached_occupancy(OccCache& cache, K* kern, int threads, size_t smem,
     return cudaSuccess;
 }
 
+// Blocks of a Dslash launch over `tiles` blocks' worth of sites: one per tile,
+// so that the hardware hands the next tile to whichever SM is free. (One
+// resident wave with a grid-stride loop gave every block the same number of
+// tiles: the average SM held 3.15 of 4 warps per scheduler; 48^3x12, n = 8,
+// FP16: 186 us, a block per tile 170.) A reduction has kMaxRedBlocks partial
+// slots: a block then takes a.run consecutive tiles, which keeps the visit
+// order that the L2 reuse rests on (strided tiles: 64^3x16, n = 4, FP32 452 us
+// against 392).
+//
+// The sums over the blocks: with many blocks, a kernel of its own after the
+// launch (launch_red_finish). Finding the last block costs every block a fence
+// over its stores and an atomic round trip while it holds its slot (32^3x8,
+// n = 8, FP32, second Dslash of the CG: 59 us against 43 without the sums).
+// Few blocks (kInlineBlocks) run side by side, and the launch costs more.
+constexpr int kInlineBlocks = 128;
+inline unsigned plan_tiles(DslashArgs& a, long long tiles) {
+    a.run = 1;
+    if (a.red_mode != RED_NONE) a.run = (int)((tiles + kMaxRedBlocks - 1) / kMaxRedBlocks);
+    const long long blocks = (tiles + a.run - 1) / a.run;
+    a.red_defer = a.red_mode != RED_NONE && blocks > kInlineBlocks;
+    return (unsigned)blocks;
+}
+inline cudaError_t finish_launch(const DslashArgs& a, unsigned blocks, cudaStream_t s) {
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess && a.red_defer ? launch_red_finish(a, (int)blocks, s) : e;
+}
+
 // ---------------------------------------------------------------------------
 // Host-side launcher for one instance
 // ---------------------------------------------------------------------------
 template <typename S, typename LS, int RU, int RN, int RPT, int MINB, int EPI, int LAYOUT, bool PACK>
-cudaError_t launch_dslash_instance(const DslashArgs& a, cudaStream_t s) {
+cudaError_t launch_dslash_instance(const DslashArgs& args, cudaStream_t s) {
+    DslashArgs a = args;
     const int G = a.nrhs / RPT;
     if (G < 1 || G * RPT != a.nrhs || G > 8) return cudaErrorInvalidValue;
     int bx = 256 / G;
@@ -597,12 +638,14 @@ cudaError_t launch_dslash_instance(const DslashArgs& a, cudaStream_t s) {
     int occ = 0;
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
-    long long nblk = ((long long)a.g.vh + bx - 1) / bx;
-    long long cap = (long long)occ * device_sm_count();
-    if (nblk > cap) nblk = cap;
-    if (nblk > kMaxRedBlocks) nblk = kMaxRedBlocks;
-    kern<<<(unsigned)nblk, block, 0, s>>>(a);
-    return cudaGetLastError();
+    // one resident wave (a block per tile: 20x28x36x10, n = 6, FP32 1 % slower)
+    long long tiles = ((long long)a.g.vh + bx - 1) / bx;
+    const long long cap = (long long)occ * device_sm_count();
+    if (tiles > cap) tiles = cap;
+    if (tiles > kMaxRedBlocks) tiles = kMaxRedBlocks;
+    const unsigned blocks = plan_tiles(a, tiles);
+    kern<<<blocks, block, 0, s>>>(a);
+    return finish_launch(a, blocks, s);
 }
 
 // Output site of the v-th visit. The sites of one (z, t) plane (an x-y block

@@ -213,8 +213,8 @@ __global__ void __launch_bounds__(256, MINB) dslash_pipe_kernel(const DslashArgs
         red0[j] = (R)0;
         red1[j] = (R)0;
     }
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v - (int)threadIdx.x < vh;
-         v += gridDim.x * blockDim.x) {
+    const int v0 = blockIdx.x * a.run * blockDim.x;
+    for (int it = 0, v = v0 + threadIdx.x; it < a.run && v - (int)threadIdx.x < vh; ++it, v += blockDim.x) {
         if (v >= vh) continue;
         const int h = visit_site(v, a.g);
         RC acc[RPT][3];
@@ -246,7 +246,8 @@ __global__ void __launch_bounds__(256, MINB) dslash_pipe_kernel(const DslashArgs
 }
 
 template <typename S, typename LS, int RU, int RN, int RPT, int MINB, int DEPTH, int EPI, int LAYOUT>
-cudaError_t launch_dslash_pipe(const DslashArgs& a, cudaStream_t s) {
+cudaError_t launch_dslash_pipe(const DslashArgs& args, cudaStream_t s) {
+    DslashArgs a = args;
     if (a.t_only) return cudaErrorInvalidValue;
     const int G = a.nrhs / RPT;
     if (G < 1 || G * RPT != a.nrhs || G > 8) return cudaErrorInvalidValue;
@@ -258,12 +259,9 @@ cudaError_t launch_dslash_pipe(const DslashArgs& a, cudaStream_t s) {
     int occ = 0;
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
-    long long nblk = ((long long)a.g.vh + bx - 1) / bx;
-    long long cap = (long long)occ * device_sm_count();
-    if (nblk > cap) nblk = cap;
-    if (nblk > kMaxRedBlocks) nblk = kMaxRedBlocks;
-    kern<<<(unsigned)nblk, block, 0, s>>>(a);
-    return cudaGetLastError();
+    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + bx - 1) / bx);
+    kern<<<blocks, block, 0, s>>>(a);
+    return finish_launch(a, blocks, s);
 }
 
 }  // namespace hisq

@@ -235,6 +235,8 @@ struct DslashArgs {
     int finish;
     double tol2;                        // FIN_RELIABLE: tol^2
     RedScratch red;
+    int run;                            // consecutive tiles a block takes (set by the launcher)
+    int red_defer;                      // 1: the blocks' sums are left to launch_red_finish (set by the launcher)
     double* red_out;                    // [vals] for FIN_STORE
     CgScalars* cg;                      // for FIN_CG_ALPHA / FIN_RELIABLE
 };
@@ -349,6 +351,8 @@ cudaError_t launch_accum_solution(const BlasArgs& a, int prec, double2* x_hi, vo
 // does not see p)
 cudaError_t launch_dot_alpha(const BlasArgs& a, int prec, const void* p, const void* Ap,
                              cudaStream_t s);
+// The sums over the nslots blocks of a Dslash launched with a.red_defer, and its finish
+cudaError_t launch_red_finish(const DslashArgs& a, int nslots, cudaStream_t s);
 // |r_hi|^2 and max|r_i| with the reliable-update finish
 cudaError_t launch_residual_norm(const BlasArgs& a, const double2* r_hi, double tol2,
                                  cudaStream_t s);

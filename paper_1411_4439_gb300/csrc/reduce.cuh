@@ -25,6 +25,33 @@ __device__ __forceinline__ R warp_max(R v) {
     return v;
 }
 
+// N per-lane values (N a power of two <= 32) reduced over the warp together:
+// every exchange halves the values a lane carries, so 8 values take 9 shuffles
+// instead of 40. The result is value multi_index<N>(lane), in all lanes that
+// agree in the top log2(N) bits of the lane number; fixed order.
+template <int N>
+__device__ __forceinline__ int multi_index(int lane) {
+    return N == 1 ? 0 : lane / (32 / N);
+}
+template <int N, typename R, typename Op>
+__device__ __forceinline__ R warp_multi(R (&v)[N], Op op) {
+    const int lane = threadIdx.x & 31;
+    int mask = 16;
+#pragma unroll
+    for (int w = N / 2; w >= 1; w >>= 1, mask >>= 1) {
+        const bool up = lane & mask;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const R send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+            v[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, mask));
+        }
+    }
+    R t = v[0];
+#pragma unroll
+    for (; mask >= 1; mask >>= 1) t = op(t, __shfl_xor_sync(0xffffffffu, t, mask));
+    return t;
+}
+
 // Signals arrival of this block; true in the block that arrived last.
 __device__ __forceinline__ bool last_block_arrive(unsigned int* counter, unsigned int nblocks) {
     __shared__ unsigned int s_last;
@@ -51,9 +78,15 @@ __device__ __forceinline__ void finish_values(const RedScratch& red, int nvals, 
         const double* src = red.partials + (size_t)v * kMaxRedBlocks;
         const bool mx = is_max(v);
         double acc = 0.0;
-        for (int i = lane; i < nslots; i += 32) {
-            const double t = __ldcg(src + i);
-            acc = mx ? fmax(acc, t) : acc + t;
+        // U loads in flight per lane: up to 4096 slots are summed while the
+        // rest of the GPU waits
+        constexpr int U = 8;
+        for (int i0 = lane; i0 < nslots; i0 += 32 * U) {
+            double t[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) t[u] = i0 + 32 * u < nslots ? __ldcg(src + i0 + 32 * u) : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc = mx ? fmax(acc, t[u]) : acc + t[u];
         }
         acc = mx ? warp_max(acc) : warp_sum(acc);
         if (lane == 0) out_smem[v] = acc;
@@ -71,87 +104,90 @@ __device__ __forceinline__ bool moving(const CgScalars* cg, int k) {
     return cg->active[k] && !cg->frozen[k];
 }
 
-// pAp -> alpha_k = rr_k / pAp_k for moving rhs. A non-finite pAp is an error;
-// pAp <= 0 means the low-precision iteration lost A-conjugacy: alpha = 0 and
-// this iteration restarts the rhs from p = r (beta = 0).
-__device__ __forceinline__ void finish_cg_alpha(CgScalars* cg, const double* vals, int n) {
-    const int k = threadIdx.x + threadIdx.y * blockDim.x;
-    if (k < n) {
-        const double pAp = vals[k];
-        double alpha = 0.0;
-        if (moving(cg, k)) {
-            if (!isfinite(pAp)) {
-                atomicOr(&cg->flags, kFlagNaN);
-            } else if (!(pAp > 0.0) || !(cg->rr[k] <= cg->alpha_max * pAp)) {
-                // pAp <= 0, or alpha above 1/lambda_min: the low-precision
-                // iteration lost conjugacy; restart this rhs from p = r
-                cg->stall[k] = 1;
-            } else {
-                alpha = cg->rr[k] / pAp;
-            }
-        }
-        cg->pAp[k] = pAp;
-        cg->alpha[k] = alpha;
-    }
-}
-
-// rr' -> beta_k = rr'_k / rr_k, rr_k = rr'_k for moving rhs; freezes an rhs
-// whose residual fell by more than freeze2 since the last reliable update.
-__device__ __forceinline__ void finish_cg_beta(CgScalars* cg, const double* vals, int n) {
-    const int k = threadIdx.x + threadIdx.y * blockDim.x;
-    if (k < n) {
-        double beta = 0.0;
-        if (moving(cg, k)) {
-            const double rr_new = vals[k];
-            if (!isfinite(rr_new)) {
-                atomicOr(&cg->flags, kFlagNaN);
-            } else {
-                if (cg->stall[k]) {
-                    cg->stall[k] = 0;
-                    cg->restarts[k] += 1;
-                } else if (cg->rr[k] > 0.0) {
-                    beta = rr_new / cg->rr[k];
-                }
-                cg->rr[k] = rr_new;
-                if (rr_new <= cg->freeze2 * cg->rr_rel[k]) cg->frozen[k] = 1;
-            }
-        }
-        cg->beta[k] = beta;
-    }
-}
-
-// FP64 true residual (|r|^2 at vals[2k], max|r_i| at vals[2k+1]): record it,
-// retire rhs whose residual meets tol2 * |b|^2, pick the next scale.
-__device__ __forceinline__ void finish_reliable(CgScalars* cg, const double* vals, int n,
-                                                double tol2) {
-    const int k = threadIdx.x + threadIdx.y * blockDim.x;
-    if (k < n) {
-        const double nrm = vals[2 * k], mx = vals[2 * k + 1];
-        // The search direction p is kept across the update while the
-        // iterated residual still describes the true one. Once the true
-        // residual is 10x (in norm) above the iterated one, the iteration has
-        // run into its rounding floor and p no longer belongs to this
-        // residual; a frozen rhs skipped its last p update. Both restart
-        // from p = r.
-        const double sc = cg->scale[k];
-        const double iterated = cg->rr[k] / (sc * sc);
-        cg->reset_p[k] = (nrm > 100.0 * iterated || cg->frozen[k]) ? 1 : 0;
-        cg->rr_true[k] = nrm;
-        cg->rmax[k] = mx;
-        const int better = isfinite(nrm) && (!cg->have_best[k] || nrm < cg->rr_best[k]);
-        cg->keep[k] = better;
-        if (better) {
-            cg->rr_best[k] = nrm;
-            cg->have_best[k] = 1;
-        }
-        if (!isfinite(nrm)) {
+// pAp -> alpha_k = rr_k / pAp_k for a moving rhs k. A non-finite pAp is an
+// error; pAp <= 0 means the low-precision iteration lost A-conjugacy: alpha = 0
+// and this iteration restarts the rhs from p = r (beta = 0).
+__device__ __forceinline__ void finish_cg_alpha(CgScalars* cg, int k, double pAp) {
+    double alpha = 0.0;
+    if (moving(cg, k)) {
+        if (!isfinite(pAp)) {
             atomicOr(&cg->flags, kFlagNaN);
-            cg->active[k] = 0;
-        } else if (cg->active[k] && nrm <= tol2 * cg->bb[k]) {
-            cg->active[k] = 0;
+        } else if (!(pAp > 0.0) || !(cg->rr[k] <= cg->alpha_max * pAp)) {
+            // pAp <= 0, or alpha above 1/lambda_min: the low-precision
+            // iteration lost conjugacy; restart this rhs from p = r
+            cg->stall[k] = 1;
+        } else {
+            alpha = cg->rr[k] / pAp;
         }
-        cg->scale_old[k] = cg->scale[k];
-        cg->scale[k] = (mx > 0.0 && isfinite(mx)) ? 1.0 / mx : 1.0;
+    }
+    cg->pAp[k] = pAp;
+    cg->alpha[k] = alpha;
+}
+
+// rr' -> beta_k = rr'_k / rr_k, rr_k = rr'_k for a moving rhs; freezes an rhs
+// whose residual fell by more than freeze2 since the last reliable update.
+__device__ __forceinline__ void finish_cg_beta(CgScalars* cg, int k, double rr_new) {
+    double beta = 0.0;
+    if (moving(cg, k)) {
+        if (!isfinite(rr_new)) {
+            atomicOr(&cg->flags, kFlagNaN);
+        } else {
+            if (cg->stall[k]) {
+                cg->stall[k] = 0;
+                cg->restarts[k] += 1;
+            } else if (cg->rr[k] > 0.0) {
+                beta = rr_new / cg->rr[k];
+            }
+            cg->rr[k] = rr_new;
+            if (rr_new <= cg->freeze2 * cg->rr_rel[k]) cg->frozen[k] = 1;
+        }
+    }
+    cg->beta[k] = beta;
+}
+
+// FP64 true residual of rhs k (|r|^2 and max |r_i|): record it, retire the rhs
+// if it meets tol2 * |b|^2, pick the next scale.
+__device__ __forceinline__ void finish_reliable(CgScalars* cg, int k, double nrm, double mx, double tol2) {
+    // The search direction p is kept across the update while the
+    // iterated residual still describes the true one. Once the true
+    // residual is 10x (in norm) above the iterated one, the iteration has
+    // run into its rounding floor and p no longer belongs to this
+    // residual; a frozen rhs skipped its last p update. Both restart
+    // from p = r.
+    const double sc = cg->scale[k];
+    const double iterated = cg->rr[k] / (sc * sc);
+    cg->reset_p[k] = (nrm > 100.0 * iterated || cg->frozen[k]) ? 1 : 0;
+    cg->rr_true[k] = nrm;
+    cg->rmax[k] = mx;
+    const int better = isfinite(nrm) && (!cg->have_best[k] || nrm < cg->rr_best[k]);
+    cg->keep[k] = better;
+    if (better) {
+        cg->rr_best[k] = nrm;
+        cg->have_best[k] = 1;
+    }
+    if (!isfinite(nrm)) {
+        atomicOr(&cg->flags, kFlagNaN);
+        cg->active[k] = 0;
+    } else if (cg->active[k] && nrm <= tol2 * cg->bb[k]) {
+        cg->active[k] = 0;
+    }
+    cg->scale_old[k] = cg->scale[k];
+    cg->scale[k] = (mx > 0.0 && isfinite(mx)) ? 1.0 / mx : 1.0;
+}
+
+// The reduced value(s) of rhs k as the finish of a reduction with nv values
+// per rhs: v0, and v1 (the maximum) with nv = 2.
+__device__ __forceinline__ void finish_rhs(int finish, CgScalars* cg, double* out, int k, int nv, double v0, double v1,
+                                           double tol2) {
+    if (finish == FIN_CG_ALPHA) {
+        finish_cg_alpha(cg, k, v0);
+    } else if (finish == FIN_CG_BETA) {
+        finish_cg_beta(cg, k, v0);
+    } else if (finish == FIN_RELIABLE) {
+        finish_reliable(cg, k, v0, v1, tol2);
+    } else if (out != nullptr) {
+        out[k * nv] = v0;
+        if (nv == 2) out[k * nv + 1] = v1;
     }
 }
 

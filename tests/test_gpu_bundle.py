@@ -378,3 +378,26 @@ def test_xy_tile_bundle_dslash_matches_oracle(gpu_lib, L, prec, minb):
                     assert rel_l2(got[k], ref[k]) < TOL[prec], (n, parity, k)
     finally:
         H.hisq_gauge_free(g)
+
+
+# blocks whose thread groups are no power of two (n = 12: three groups of four
+# rhs), reductions over few blocks (finished in the kernel) and many (in a
+# kernel of their own); bound: the solve's own tolerance with the oracle's residual
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("L,n", [((4, 6, 8, 10), 12), ((16, 12, 10, 14), 12), ((16, 12, 10, 14), 16), ((16, 16, 12, 12), 8)])
+def test_reductions_of_odd_groups_and_many_blocks(gpu_lib, prec, L, n):
+    import torch
+    H = gpu_lib
+    U, N = gen.hisq_links(L, seed=3)
+    m = 0.2
+    g = H.hisq_gauge_load(L, torch.from_numpy(U).cuda(), torch.from_numpy(N).cuda(), prec=prec, recon_U=18, recon_N=14)
+    try:
+        b = gen.gaussian_source(L, n, seed=4)
+        bt = [torch.from_numpy(b[k]).cuda() for k in range(n)]
+        xt = [torch.zeros_like(t) for t in bt]
+        stats = H.hisq_cg_solve(g, m, 0.0, bt, xt, 1e-10, H.cg_params(inner_prec=prec))
+        x = np.stack([t.cpu().numpy() for t in xt])
+        res = O.true_relative_residual(lambda q: O.apply_Ae(U, N, q, L, m), x, b)
+        assert np.all(res <= 1e-10) and stats.total_iters < 400
+    finally:
+        H.hisq_gauge_free(g)
