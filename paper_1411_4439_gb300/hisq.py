@@ -150,9 +150,20 @@ def _check(status: int, stats=None):
 # marshalling helpers
 # ---------------------------------------------------------------------------
 
+# A small call's time is this marshalling (8^4 Dslash of one vector: 29 us of
+# host work with a torch Stream object and per-element array stores a call for
+# a kernel of a few us), hence the raw stream handle and one array constructor.
+
+_torch_mod = None
+_raw_stream = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod
+    if _torch_mod is None:
+        import torch
+        _torch_mod = torch
+    return _torch_mod
 
 
 def _ptr(buf) -> int:
@@ -171,22 +182,31 @@ def _ptr(buf) -> int:
 
 
 def _is_device(buf) -> bool:
-    return hasattr(buf, "is_cuda") and bool(buf.is_cuda)
+    return bool(getattr(buf, "is_cuda", False))
+
+
+def _current_stream() -> int:
+    """Handle of torch's current stream on the current device."""
+    global _raw_stream
+    torch = _torch()
+    if _raw_stream is None:
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", False)
+    if _raw_stream:
+        return int(_raw_stream(torch.cuda.current_device()))
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 def _stream_handle(stream, *bufs) -> int | None:
     if stream is not None:
         return int(getattr(stream, "cuda_stream", stream))
-    if any(_is_device(b) for b in bufs):
-        return int(_torch().cuda.current_stream().cuda_stream)
+    for b in bufs:
+        if _is_device(b):
+            return _current_stream()
     return None
 
 
 def _ptr_array(bufs):
-    arr = (ctypes.c_void_p * len(bufs))()
-    for i, b in enumerate(bufs):
-        arr[i] = _ptr(b)
-    return arr
+    return (ctypes.c_void_p * len(bufs))(*[_ptr(b) for b in bufs])
 
 
 def _lattice(L):
@@ -397,12 +417,15 @@ def _check_fp64_vectors(vs):
     torch = _torch()
     if len(vs) == 0:
         raise ValueError("no vectors")
+    first = vs[0]
+    if _is_device(first):
+        dtype, device, numel = first.dtype, first.device, first.numel()
     for t in vs:
-        if not hasattr(t, "is_cuda") or not t.is_cuda:
+        if not _is_device(t):
             raise ValueError("vectors must be CUDA tensors")
         if t.dtype not in (torch.complex128, torch.float64):
             raise ValueError(f"vectors must be complex128 or float64, got {t.dtype}")
-        if t.dtype != vs[0].dtype or t.device != vs[0].device or t.numel() != vs[0].numel():
+        if t.dtype != dtype or t.device != device or t.numel() != numel:
             raise ValueError("vectors must share dtype, device and length")
 
 
