@@ -164,20 +164,21 @@ enum {
     HISQ_MAP_TILE_XY = 256
 };
 /* On the bundle layout (rhs per thread 4 or 8, min blocks per SM of 128-thread
- * blocks 1..4) the kernel multiplies rhs pairs with packed FP32 (f32x2)
+ * blocks 1..6) the kernel multiplies rhs pairs with packed FP32 (f32x2)
  * instructions and keeps the next hop's link load in flight; flags select
  * variants: HISQ_MAP_PIPELINED also the next hop's neighbour chunks,
  * HISQ_MAP_COMPACT a hop loop with the direction as a runtime loop (a quarter
  * of the code, one colour of the neighbours converted at a time),
  * HISQ_MAP_STAGED the neighbour chunks copied into shared memory by
  * asynchronous per-thread copies one hop ahead (two with HISQ_MAP_PIPELINED2;
- * together with HISQ_MAP_COMPACT one, or three with HISQ_MAP_PIPELINED2).
+ * together with HISQ_MAP_COMPACT one, or three with HISQ_MAP_PIPELINED2, and
+ * the links with them).
  * HISQ_MAP_TILE_XY the neighbours of the x and y hops read from a
  * shared-memory tile of whole x-rows of the block's (z, t) plane (loaded while
  * the z and t hops run; one rhs group, i.e. n equal to rhs per thread, and
  * planes of whole 128-site runs, else the plain loop).
- * Defaults at 8 rhs per thread: FP16 storage STAGED | COMPACT at 4 blocks per
- * SM, FP32 storage no flag at 3 blocks per SM. */
+ * Defaults: FP16 storage STAGED | COMPACT at 4 blocks per SM with 8 rhs per
+ * thread and 6 with 4, FP32 storage no flag at 3 and 4 blocks per SM. */
 hisq_status hisq_set_dslash_mapping(hisq_gauge g, int rhs_per_thread, int min_blocks,
                                     int flags);
 

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kThreads) update_r_kernel(BlasArgs a, void* r,
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[1] = {false};
     if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
-        finish_cg_beta(a.cg, threadIdx.x, s_vals[threadIdx.x]);
+        finish_cg_beta(a.cg, threadIdx.x, s_vals[threadIdx.x], fin_load(a.cg, threadIdx.x));
 }
 
 // x += alpha p ; p = r + beta p, both from the old p, in one pass. alpha is
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kThreads) dot_alpha_kernel(BlasArgs a, const v
     __shared__ double s_vals[kMaxRedVals];
     const bool mx[1] = {false};
     if (block_reduce_arrive<R, 1>(a.red, val, a.n, mx, s_vals) && threadIdx.x < a.n)
-        finish_cg_alpha(a.cg, threadIdx.x, s_vals[threadIdx.x]);
+        finish_cg_alpha(a.cg, threadIdx.x, s_vals[threadIdx.x], fin_load(a.cg, threadIdx.x));
 }
 
 // |r_hi|^2 and max |r_i| -> reliable finish (full-lattice residual)
@@ -416,21 +416,30 @@ __global__ void __launch_bounds__(kThreads) residual_norm_kernel(BlasArgs a, con
         finish_reliable(a.cg, threadIdx.x, s_vals[2 * threadIdx.x], s_vals[2 * threadIdx.x + 1], tol2);
 }
 
-// Sums of a reduction over its nslots blocks, one block per rhs, and the finish.
-__global__ void __launch_bounds__(kThreads) red_finish_kernel(RedScratch red, int nslots, int nv, int finish,
-                                                              CgScalars* cg, double* out, double tol2) {
+// Sums of a reduction over its nslots blocks, one block per rhs, and the
+// finish. It is pure latency between two Dslash-sized kernels: the scalars the
+// finish needs are loaded beside the partial sums, and no thread adds zeros (a
+// warp's FP64 add takes the SM 16 cycles; 512 threads with 8 slots each, most
+// of them empty at 1024 slots, took 2.5 us more).
+constexpr int kFinishThreads = 256;
+__global__ void __launch_bounds__(kFinishThreads) red_finish_kernel(RedScratch red, int nslots, int nv, int finish,
+                                                                    CgScalars* cg, double* out, double tol2) {
     const int k = blockIdx.x;
-    __shared__ double s_w[2][kThreads / 32];
+    __shared__ double s_w[2][kFinishThreads / 32];
+    FinState st;
+    if (threadIdx.x == 0 && finish != FIN_STORE) st = fin_load(cg, k);
     for (int j = 0; j < nv; ++j) {
-        const double* src = red.partials + (size_t)(k * nv + j) * kMaxRedBlocks;
+        const double* src = red.partials + (size_t)(k * nv + j) * kDeferSlots;
         constexpr int U = 4;
         double acc = 0.0;
-        for (int i0 = threadIdx.x; i0 < nslots; i0 += U * kThreads) {
+        for (int i0 = threadIdx.x; i0 < nslots; i0 += U * kFinishThreads) {
             double t[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) t[u] = i0 + u * kThreads < nslots ? __ldcg(src + i0 + u * kThreads) : 0.0;
+            for (int u = 0; u < U; ++u)
+                if (i0 + u * kFinishThreads < nslots) t[u] = __ldcg(src + i0 + u * kFinishThreads);
 #pragma unroll
-            for (int u = 0; u < U; ++u) acc = j ? fmax(acc, t[u]) : acc + t[u];
+            for (int u = 0; u < U; ++u)
+                if (i0 + u * kFinishThreads < nslots) acc = j ? fmax(acc, t[u]) : acc + t[u];
         }
         acc = j ? warp_max(acc) : warp_sum(acc);
         if ((threadIdx.x & 31) == 0) s_w[j][threadIdx.x >> 5] = acc;
@@ -438,11 +447,12 @@ __global__ void __launch_bounds__(kThreads) red_finish_kernel(RedScratch red, in
     __syncthreads();
     if (threadIdx.x == 0) {
         double v0 = 0.0, v1 = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
+#pragma unroll
+        for (int w = 0; w < kFinishThreads / 32; ++w) {
             v0 += s_w[0][w];
             if (nv == 2) v1 = fmax(v1, s_w[1][w]);
         }
-        finish_rhs(finish, cg, out, k, nv, v0, v1, tol2);
+        finish_rhs(finish, cg, out, k, nv, v0, v1, tol2, st);
     }
 }
 
@@ -523,7 +533,7 @@ cudaError_t launch_dot_alpha(const BlasArgs& a, int prec, const void* p, const v
 
 cudaError_t launch_red_finish(const DslashArgs& a, int nslots, cudaStream_t s) {
     const int nv = a.red_mode == RED_NORM_MAX_W ? 2 : 1;
-    red_finish_kernel<<<a.nrhs, kThreads, 0, s>>>(a.red, nslots, nv, a.finish, a.cg, a.red_out, a.tol2);
+    red_finish_kernel<<<a.nrhs, kFinishThreads, 0, s>>>(a.red, nslots, nv, a.finish, a.cg, a.red_out, a.tol2);
     return cudaGetLastError();
 }
 

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 4) update_r_b_kernel(BlasArgs a, uin
     }
     __shared__ double s_vals[kMaxRedVals];
     if (group_reduce_arrive<W>(a.red, val, gridDim.y, s_vals) && threadIdx.x < a.n)
-        finish_cg_beta(a.cg, threadIdx.x, s_vals[threadIdx.x]);
+        finish_cg_beta(a.cg, threadIdx.x, s_vals[threadIdx.x], fin_load(a.cg, threadIdx.x));
 }
 
 // x_lo += alpha p ; p = r + beta p (moving rhs), both from the old p.

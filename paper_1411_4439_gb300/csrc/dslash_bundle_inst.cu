@@ -32,6 +32,7 @@ static cudaError_t bundle_by_variant(const DslashArgs& a, int rpt, int minb, int
         case 4405: return HISQ_B(4, 4, 0, false);
         case 8309: return HISQ_B(8, 3, 0, true);
         case 8413: return HISQ_BS(8, 4, 11);
+        case 4613: return HISQ_BS(4, 6, 11);
 #if HISQ_BUNDLE_FULL
         case 8205: return HISQ_B(8, 2, 0, false);
         case 4305: return HISQ_B(4, 3, 0, false);

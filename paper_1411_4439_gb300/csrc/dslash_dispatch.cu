@@ -46,7 +46,7 @@ int dslash_max_rpt(int prec) { return prec == HISQ_F64 ? 4 : 8; }
 bool bundle_mapping_built(int prec, int ru, int rn, int rpt, int minb, int kind) {
     if (prec != HISQ_F32 && prec != HISQ_F16) return false;
     const int key = rpt * 1000 + minb * 100 + kind;
-    if (key == 8305 || key == 4405 || key == 8309 || key == 8413) return true;
+    if (key == 8305 || key == 4405 || key == 8309 || key == 8413 || key == 4613) return true;
     if (!(ru == 18 && rn == 14)) return false;
     switch (key) {
         case 8205: case 4305: case 4409: case 8105: case 8106: case 8206: case 4306: case 8209: case 8409: case 4309:
@@ -61,8 +61,11 @@ bool bundle_mapping_built(int prec, int ru, int rn, int rpt, int minb, int kind)
 // Default bundle mapping for n rhs: eight rhs per thread when n allows
 // (every link element then serves four rhs pairs), else four. Measured at
 // 48^3x12, n = 8: FP16 storage runs fastest with the compact hop loop and
-// the neighbour chunks staged in shared memory (16 warps per SM, 201 us),
-// FP32 with the unrolled loop at 12 warps per SM (215 us).
+// the neighbour chunks and links staged in shared memory (16 warps per SM,
+// 170 us), FP32 with the unrolled loop at 12 warps per SM (195 us). Four rhs
+// per thread, FP16, 64^3x16, n = 4: that loop at 24 warps per SM 309 us (338
+// at 16, unrolled loop 340); FP32 the unrolled loop (386 us, 98 % of the
+// measured HBM rate).
 DslashTune dslash_bundle_tune(int prec, int n) {
     DslashTune t;
     t.layout = HISQ_BUNDLE;
@@ -78,7 +81,8 @@ DslashTune dslash_bundle_tune(int prec, int n) {
         if (prec == HISQ_F16) t.kind = KIND_BUNDLE_CSMEM1;
     } else if (n % 4 == 0 && n / 4 <= 4) {
         t.rpt = 4;
-        t.minb = 4;
+        t.minb = prec == HISQ_F16 ? 6 : 4;
+        if (prec == HISQ_F16) t.kind = KIND_BUNDLE_CSMEM1;
     }
     return t;
 }

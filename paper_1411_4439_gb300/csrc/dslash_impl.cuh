@@ -523,13 +523,14 @@ __device__ __forceinline__ void block_finish(const DslashArgs& a, const RedParts
         const bool is_max = (nv == 2) && (tid & 1);
         double acc = 0.0;
         for (int w = 0; w < wpg; ++w) acc = is_max ? fmax(acc, parts.v[tid][w]) : acc + parts.v[tid][w];
-        a.red.partials[(size_t)tid * kMaxRedBlocks + blockIdx.x] = acc;
+        a.red.partials[(size_t)tid * (a.red_defer ? kDeferSlots : kMaxRedBlocks) + blockIdx.x] = acc;
     }
     if (a.red_defer) return;
     if (!last_block_arrive(a.red.counter, gridDim.x)) return;
     finish_values(a.red, nvals, gridDim.x, [nv](int v) { return nv == 2 && (v & 1); }, s_vals);
     if (tid < a.nrhs)
-        finish_rhs(a.finish, a.cg, a.red_out, tid, nv, s_vals[tid * nv], nv == 2 ? s_vals[tid * nv + 1] : 0.0, a.tol2);
+        finish_rhs(a.finish, a.cg, a.red_out, tid, nv, s_vals[tid * nv], nv == 2 ? s_vals[tid * nv + 1] : 0.0, a.tol2,
+                   fin_load(a.cg, tid));
 }
 
 template <int RPT, typename R>
@@ -599,8 +600,8 @@ cudaError_t cached_occupancy(OccCache& cache, K* kern, int threads, size_t smem,
 // so that the hardware hands the next tile to whichever SM is free. (One
 // resident wave with a grid-stride loop gave every block the same number of
 // tiles: the average SM held 3.15 of 4 warps per scheduler; 48^3x12, n = 8,
-// FP16: 186 us, a block per tile 170.) A reduction has kMaxRedBlocks partial
-// slots: a block then takes a.run consecutive tiles, which keeps the visit
+// FP16: 186 us, a block per tile 170.) A reduction has kDeferSlots partial
+// slots: beyond, a block takes a.run consecutive tiles, which keeps the visit
 // order that the L2 reuse rests on (strided tiles: 64^3x16, n = 4, FP32 452 us
 // against 392).
 //
@@ -612,7 +613,7 @@ cudaError_t cached_occupancy(OccCache& cache, K* kern, int threads, size_t smem,
 constexpr int kInlineBlocks = 128;
 inline unsigned plan_tiles(DslashArgs& a, long long tiles) {
     a.run = 1;
-    if (a.red_mode != RED_NONE) a.run = (int)((tiles + kMaxRedBlocks - 1) / kMaxRedBlocks);
+    if (a.red_mode != RED_NONE) a.run = (int)((tiles + kDeferSlots - 1) / kDeferSlots);
     const long long blocks = (tiles + a.run - 1) / a.run;
     a.red_defer = a.red_mode != RED_NONE && blocks > kInlineBlocks;
     return (unsigned)blocks;

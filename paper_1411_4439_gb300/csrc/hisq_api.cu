@@ -551,9 +551,11 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
         const int ru = link_recon_u(g, prec), rn = link_recon_n(g, prec);
         const int r = requested ? requested : g->tune_rpt;
         if (r && n % r == 0 && n / r <= 4) {
-            const int b = (!requested && g->tune_minb) ? g->tune_minb : (r == 8 && prec != HISQ_F16 ? 3 : 4);
-            const int k = requested ? (r == 8 && prec == HISQ_F16 ? KIND_BUNDLE_CSMEM1 : KIND_BUNDLE)
-                                    : bundle_kind_of_flags(g->tune_flags);
+            const bool f16 = prec == HISQ_F16;
+            const int b = (!requested && g->tune_minb) ? g->tune_minb
+                          : r == 8                      ? (f16 ? 4 : 3)
+                                                        : (requested && f16 ? 6 : 4);
+            const int k = requested ? (f16 ? KIND_BUNDLE_CSMEM1 : KIND_BUNDLE) : bundle_kind_of_flags(g->tune_flags);
             if (bundle_mapping_built(prec, ru, rn, r, b, k)) {
                 t.rpt = r;
                 t.minb = b;
@@ -801,7 +803,7 @@ std::vector<DslashTune> candidate_tunes(hisq_gauge g, int n, int prec, int layou
                              KIND_BUNDLE_XY};
         for (int r : {4, 8}) {
             if (n % r != 0 || n / r > 4) continue;
-            for (int b = 1; b <= 4; ++b)
+            for (int b = 1; b <= 6; ++b)
                 for (int k : kinds) {
                     if (!bundle_mapping_built(prec, ru, rn, r, b, k)) continue;
                     DslashTune t = dslash_bundle_tune(prec, n);
@@ -1178,7 +1180,7 @@ hisq_status get_workspace(hisq_gauge g, int n, int prec, int full, Workspace** o
     al((void**)&w->t_hi, thi);
     al((void**)&w->x_best, hi);
     al((void**)&w->cg, sizeof(CgScalars));
-    al((void**)&w->partials, sizeof(double) * kMaxRedVals * kMaxRedBlocks);
+    al((void**)&w->partials, sizeof(double) * kMaxRedVals * std::max(kMaxRedBlocks, kDeferSlots));
     al((void**)&w->counter, sizeof(unsigned int) * 4);
     if (e == cudaSuccess) e = cudaMemset(w->counter, 0, sizeof(unsigned int) * 4);
     // vectors of rhs that never iterate must still hold finite numbers

@@ -17,7 +17,8 @@ namespace hisq {
 
 constexpr int kMaxRhs = 16;
 constexpr int kMaxRedVals = 2 * kMaxRhs;   // per-rhs norm and max
-constexpr int kMaxRedBlocks = 4096;         // partial-sum slots per reduction
+constexpr int kMaxRedBlocks = 4096;         // partial-sum slots per reduction finished by its last block
+constexpr int kDeferSlots = 16384;          // ... and per Dslash reduction finished by a kernel of its own
 
 // ---------------------------------------------------------------------------
 // Geometry of the checkerboarded lattice

@@ -104,20 +104,39 @@ __device__ __forceinline__ bool moving(const CgScalars* cg, int k) {
     return cg->active[k] && !cg->frozen[k];
 }
 
+// The scalars of rhs k that the finishes read, loaded together (one latency
+// instead of one for each that follows a branch).
+struct FinState {
+    int moves, stall;
+    double rr, rr_rel, freeze2, alpha_max;
+};
+__device__ __forceinline__ FinState fin_load(const CgScalars* cg, int k) {
+    FinState f;
+    if (cg == nullptr) return f;
+    const int act = cg->active[k], frz = cg->frozen[k];
+    f.stall = cg->stall[k];
+    f.rr = cg->rr[k];
+    f.rr_rel = cg->rr_rel[k];
+    f.freeze2 = cg->freeze2;
+    f.alpha_max = cg->alpha_max;
+    f.moves = act && !frz;
+    return f;
+}
+
 // pAp -> alpha_k = rr_k / pAp_k for a moving rhs k. A non-finite pAp is an
 // error; pAp <= 0 means the low-precision iteration lost A-conjugacy: alpha = 0
 // and this iteration restarts the rhs from p = r (beta = 0).
-__device__ __forceinline__ void finish_cg_alpha(CgScalars* cg, int k, double pAp) {
+__device__ __forceinline__ void finish_cg_alpha(CgScalars* cg, int k, double pAp, const FinState& f) {
     double alpha = 0.0;
-    if (moving(cg, k)) {
+    if (f.moves) {
         if (!isfinite(pAp)) {
             atomicOr(&cg->flags, kFlagNaN);
-        } else if (!(pAp > 0.0) || !(cg->rr[k] <= cg->alpha_max * pAp)) {
+        } else if (!(pAp > 0.0) || !(f.rr <= f.alpha_max * pAp)) {
             // pAp <= 0, or alpha above 1/lambda_min: the low-precision
             // iteration lost conjugacy; restart this rhs from p = r
             cg->stall[k] = 1;
         } else {
-            alpha = cg->rr[k] / pAp;
+            alpha = f.rr / pAp;
         }
     }
     cg->pAp[k] = pAp;
@@ -126,20 +145,20 @@ __device__ __forceinline__ void finish_cg_alpha(CgScalars* cg, int k, double pAp
 
 // rr' -> beta_k = rr'_k / rr_k, rr_k = rr'_k for a moving rhs; freezes an rhs
 // whose residual fell by more than freeze2 since the last reliable update.
-__device__ __forceinline__ void finish_cg_beta(CgScalars* cg, int k, double rr_new) {
+__device__ __forceinline__ void finish_cg_beta(CgScalars* cg, int k, double rr_new, const FinState& f) {
     double beta = 0.0;
-    if (moving(cg, k)) {
+    if (f.moves) {
         if (!isfinite(rr_new)) {
             atomicOr(&cg->flags, kFlagNaN);
         } else {
-            if (cg->stall[k]) {
+            if (f.stall) {
                 cg->stall[k] = 0;
                 cg->restarts[k] += 1;
-            } else if (cg->rr[k] > 0.0) {
-                beta = rr_new / cg->rr[k];
+            } else if (f.rr > 0.0) {
+                beta = rr_new / f.rr;
             }
             cg->rr[k] = rr_new;
-            if (rr_new <= cg->freeze2 * cg->rr_rel[k]) cg->frozen[k] = 1;
+            if (rr_new <= f.freeze2 * f.rr_rel) cg->frozen[k] = 1;
         }
     }
     cg->beta[k] = beta;
@@ -178,11 +197,11 @@ __device__ __forceinline__ void finish_reliable(CgScalars* cg, int k, double nrm
 // The reduced value(s) of rhs k as the finish of a reduction with nv values
 // per rhs: v0, and v1 (the maximum) with nv = 2.
 __device__ __forceinline__ void finish_rhs(int finish, CgScalars* cg, double* out, int k, int nv, double v0, double v1,
-                                           double tol2) {
+                                           double tol2, const FinState& f) {
     if (finish == FIN_CG_ALPHA) {
-        finish_cg_alpha(cg, k, v0);
+        finish_cg_alpha(cg, k, v0, f);
     } else if (finish == FIN_CG_BETA) {
-        finish_cg_beta(cg, k, v0);
+        finish_cg_beta(cg, k, v0, f);
     } else if (finish == FIN_RELIABLE) {
         finish_reliable(cg, k, v0, v1, tol2);
     } else if (out != nullptr) {
