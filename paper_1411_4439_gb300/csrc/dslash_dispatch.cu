@@ -178,7 +178,7 @@ static cudaError_t launch_bundle(const DslashArgs& a, int prec, int ru, int rn, 
 // (8^4, n = 1: 14.7 us with one lane, 8.3 with four; 16^4, n = 1, where every
 // scheduler has one or two: 24.6 and 31).
 static int fx64_split(const DslashArgs& a, int rpt) {
-    const long long warps = ((long long)a.g.vh * (a.nrhs / rpt) + 31) / 32;
+    const long long warps = ((a.both ? 2ll : 1ll) * a.g.vh * (a.nrhs / rpt) + 31) / 32;
     return rpt <= 2 && warps < 4ll * device_sm_count() ? 4 : 1;
 }
 
@@ -198,6 +198,7 @@ cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi
         return launch_dslash(c, prec, ru, rn, epi, t, s);
     }
     const int r = t.rpt, b = t.minb, k = t.kind, l = t.layout;
+    if (a.both && !dslash_both_ok(a, prec)) return cudaErrorInvalidValue;
     if (prec == HISQ_F64 && a.fx) {
         const int split = fx64_split(a, r);
         return l == HISQ_SOA ? dslash_fx64_soa(a, epi, r, split, s) : dslash_fx64_aos(a, epi, r, split, s);

@@ -1039,10 +1039,11 @@ extern "C" hisq_status hisq_apply_m(hisq_gauge g, double mass, double mu, int op
     for (int par = 0; par < 2; ++par) {
         DslashArgs a;
         fill_common(a, g, spinor_prec, par, n);
+        a.both = dslash_both_ok(a, spinor_prec);
         for (int k = 0; k < n; ++k) {
-            a.in[k] = (const char*)v[k] + (1 - par) * half;
-            a.out[k] = (char*)w[k] + par * half;
-            a.x[k] = (const char*)v[k] + par * half;
+            a.in[k] = (const char*)v[k] + (a.both ? 0 : (1 - par) * half);
+            a.out[k] = (char*)w[k] + (a.both ? 0 : par * half);
+            a.x[k] = (const char*)v[k] + (a.both ? 0 : par * half);
         }
         int epi = EPI_X;
         if (op == HISQ_OP_M) {
@@ -1068,6 +1069,7 @@ extern "C" hisq_status hisq_apply_m(hisq_gauge g, double mass, double mu, int op
             epi = EPI_NONE;
         }
         HISQ_CUDA(launch_dslash(a, spinor_prec, ru, rn, epi, t, s));
+        if (a.both) break;
     }
     return HISQ_OK;
 }
@@ -1383,13 +1385,16 @@ struct Solver {
             set_mu(a, mu);
             a.cx = 2.0 * mass;
             a.cd = 1.0;
+            a.both = dslash_both_ok(a, prec);
+            const long long in = a.both ? 0 : (1 - par) * hl, out = a.both ? 0 : par * hl;
             for (int k = 0; k < n; ++k) {
-                a.in[k] = lo_ptr(w->p_lo, k, (1 - par) * hl);
-                a.out[k] = lo_ptr(w->t_lo, k, par * hl);
-                a.x[k] = lo_ptr(w->p_lo, k, par * hl);
+                a.in[k] = lo_ptr(w->p_lo, k, in);
+                a.out[k] = lo_ptr(w->t_lo, k, out);
+                a.x[k] = lo_ptr(w->p_lo, k, out);
             }
             e = launch_dslash(a, prec, ru, rn, EPI_X, tune, s);
             if (e != cudaSuccess) return e;
+            if (a.both) break;
         }
         if (mid) {
             e = cudaEventRecord(mid, s);
@@ -1400,13 +1405,16 @@ struct Solver {
             set_mu(a, -mu);
             a.cx = 2.0 * mass;
             a.cd = -1.0;
+            a.both = dslash_both_ok(a, prec);
+            const long long in = a.both ? 0 : (1 - par) * hl, out = a.both ? 0 : par * hl;
             for (int k = 0; k < n; ++k) {
-                a.in[k] = lo_ptr(w->t_lo, k, (1 - par) * hl);
-                a.out[k] = lo_ptr(w->Ap_lo, k, par * hl);
-                a.x[k] = lo_ptr(w->t_lo, k, par * hl);
+                a.in[k] = lo_ptr(w->t_lo, k, in);
+                a.out[k] = lo_ptr(w->Ap_lo, k, out);
+                a.x[k] = lo_ptr(w->t_lo, k, out);
             }
             e = launch_dslash(a, prec, ru, rn, EPI_X, tune, s);
             if (e != cudaSuccess) return e;
+            if (a.both) break;
         }
         return launch_dot_alpha(blas(), prec, w->p_lo, w->Ap_lo, s);
     }
@@ -1461,27 +1469,33 @@ struct Solver {
             set_mu(a, mu);
             a.cx = 2.0 * mass;
             a.cd = 1.0;
+            a.both = dslash_both_ok(a, f);
+            const long long in = a.both ? 0 : (1 - par) * hl, out = a.both ? 0 : par * hl;
             for (int k = 0; k < n; ++k) {
-                a.in[k] = hi_ptr(w->x_hi, k, (1 - par) * hl);
-                a.out[k] = hi_ptr(w->t_hi, k, par * hl);
-                a.x[k] = hi_ptr(w->x_hi, k, par * hl);
+                a.in[k] = hi_ptr(w->x_hi, k, in);
+                a.out[k] = hi_ptr(w->t_hi, k, out);
+                a.x[k] = hi_ptr(w->x_hi, k, out);
             }
             e = launch_dslash(a, f, 18, 18, EPI_X, tune64, s);
             if (e != cudaSuccess) return e;
+            if (a.both) break;
         }
         for (int par = 0; par < 2; ++par) {   // r = b - 2m y + D(-mu) y
             DslashArgs a = args(par, f);
             set_mu(a, -mu);
             a.cx = -2.0 * mass;
             a.cd = 1.0;
+            a.both = dslash_both_ok(a, f);
+            const long long in = a.both ? 0 : (1 - par) * hl, out = a.both ? 0 : par * hl;
             for (int k = 0; k < n; ++k) {
-                a.in[k] = hi_ptr(w->t_hi, k, (1 - par) * hl);
-                a.out[k] = hi_ptr(w->r_hi, k, par * hl);
-                a.x[k] = hi_ptr(w->t_hi, k, par * hl);
-                a.y[k] = hi_ptr(w->b_hi, k, par * hl);
+                a.in[k] = hi_ptr(w->t_hi, k, in);
+                a.out[k] = hi_ptr(w->r_hi, k, out);
+                a.x[k] = hi_ptr(w->t_hi, k, out);
+                a.y[k] = hi_ptr(w->b_hi, k, out);
             }
             e = launch_dslash(a, f, 18, 18, EPI_XY, tune64, s);
             if (e != cudaSuccess) return e;
+            if (a.both) break;
         }
         return launch_residual_norm(blas(), w->r_hi, tol2, s);
     }

@@ -212,6 +212,8 @@ enum Finish : int {
 struct DslashArgs {
     Geom g;
     int parity;                         // output parity
+    int both;                           // 1: both parities in one launch (F64 fixed-point links, no reduction):
+                                        // in, out, x, y are parity-blocked full-lattice vectors
     int nrhs;                           // rhs in this launch
     const void* U;                      // packed links, [2][4][ncomp][vh]
     const void* N;
@@ -282,6 +284,8 @@ DslashTune dslash_default_tune(int prec, int rpt, int layout);
 DslashTune dslash_register_tune(int prec, int rpt, int layout);
 // Whether the staged-link kernel can run this lattice with `groups` groups of rpt rhs.
 bool dslash_staged_ok(const Geom& g, int prec, int rpt, int groups);
+// Whether a launch takes both parities at once (DslashArgs::both).
+inline bool dslash_both_ok(const DslashArgs& a, int prec) { return prec == HISQ_F64 && a.fx && a.red_mode == RED_NONE; }
 // Largest rhs-per-thread value instantiated for a precision.
 int dslash_max_rpt(int prec);
 // Bundle layout: rhs per 16-byte chunk of a storage precision (F32: 2,

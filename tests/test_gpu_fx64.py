@@ -89,3 +89,29 @@ def test_links_of_different_size_and_large_factors(gpu_lib, mu):
     for links in (U, V):
         ref = O.dslash_parity(links, N, v, L, 0, mu)
         assert site_error(dslash(gpu_lib, L, links, N, v, 0, mu), ref) < 1e-13
+
+
+# both parities in one launch: every operator, in place of two launches; bound as above
+@pytest.mark.parametrize("L,n", [((4, 4, 4, 6), 1), ((4, 6, 10, 8), 3), ((12, 12, 10, 14), 4)])
+def test_full_lattice_operators_take_both_parities(gpu_lib, L, n):
+    import torch
+    H = gpu_lib
+    U, N = gen.hisq_links(L, seed=11)
+    m, mu = 0.07, 0.15
+    g = H.hisq_gauge_load(L, torch.from_numpy(U).cuda(), torch.from_numpy(N).cuda(), prec=H.HISQ_F64)
+    try:
+        rng = np.random.default_rng(12)
+        V = int(np.prod(L))
+        v = rng.standard_normal((n, V, 3)) + 1j * rng.standard_normal((n, V, 3))
+        vd = [torch.from_numpy(v[k]).cuda() for k in range(n)]
+        halves = (v[:, :V // 2], v[:, V // 2:])
+        for op, sgn, muf, mass in ((H.HISQ_OP_M, 1.0, mu, m), (H.HISQ_OP_MDAG, -1.0, -mu, m)):
+            wd = [torch.full_like(t, float("nan")) for t in vd]
+            H.hisq_apply_m(g, m, mu, op, vd, wd, H.HISQ_F64)
+            torch.cuda.synchronize()
+            for p in (0, 1):
+                ref = 2 * mass * halves[p] + sgn * O.dslash_parity(U, N, halves[1 - p], L, p, muf)
+                got = np.stack([t.cpu().numpy()[p * (V // 2):(p + 1) * (V // 2)] for t in wd])
+                assert site_error(got, ref) < 1e-13
+    finally:
+        H.hisq_gauge_free(g)
