@@ -28,11 +28,13 @@
 // What bounds it: the register ports. An IMAD.WIDE with fresh operands (two
 // factors, a 64-bit accumulator read and written) takes 3.3 to 4.2 cycles of
 // a scheduler instead of 2; the 108 of a hop and rhs are 57 % of the time, the
-// limb splitting 14 %, the rest link loads, addresses and the E test. Four
-// rhs a thread need 255 registers (8 warps a SM) and lose to two at 168.
-// Time per launch, FMA kernel -> this one: 48^3x12, n = 8: 5.24 -> 1.89 ms;
-// 64^3x16, n = 4: 8.09 -> 3.00 ms; 32^3x8, n = 8: 1055 -> 373 us; 24^3x6, n =
-// 4: 305 -> 72 us; 16^4, n = 4: 156 -> 58 us; 8^4, n = 1: 45 -> 11 us.
+// limb splitting 14 %, the rest link loads, addresses and the E test. One rhs
+// a thread at 16 warps per SM is as fast as two at 12 (48^3x12, n = 8: 1.79 and
+// 1.78 ms) or faster (32^3x8, n = 4: 178 us against 191); four need 255
+// registers (8 warps a SM) and lose.
+// Time per launch, FMA kernel -> this one: 48^3x12, n = 8: 5.24 -> 1.79 ms;
+// 32^3x8, n = 8: 1055 -> 361 us; 24^3x6, n = 4: 305 -> 68 us; 16^4, n = 4: 156
+// -> 52 us; 8^4, n = 1: 45 -> 8 us.
 //
 // E starts one above the first neighbour's largest exponent and grows when a
 // later neighbour exceeds it; the accumulators are then shifted (rounded).
@@ -233,13 +235,17 @@ struct FxHops {
             for (int i = 0; i < 3; ++i) big = max(big, max(cur[j][i].y << 1, cur[j][i].w << 1));
             nz[j] |= big;
             const int en = (int)(big >> 21) - 1022 + o;
-            if (en > E[j]) {
-                const int d = en + kFxHead - E[j];
-                E[j] = en + kFxHead;
+            // the vote keeps the branch uniform: most hops skip it without the
+            // divergence bookkeeping of a lane-wise branch (9 % of the kernel)
+            if (__any_sync(__activemask(), en > E[j])) {
+                if (en > E[j]) {
+                    const int d = en + kFxHead - E[j];
+                    E[j] = en + kFxHead;
 #pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    s2[j][i] = fx_shift(s2[j][i], d);
-                    s1[j][i] = fx_shift(s1[j][i], d);
+                    for (int i = 0; i < 6; ++i) {
+                        s2[j][i] = fx_shift(s2[j][i], d);
+                        s1[j][i] = fx_shift(s1[j][i], d);
+                    }
                 }
             }
             const int k = E[j] - o + 1030;

@@ -480,13 +480,9 @@ namespace {
 int link_recon_u(hisq_gauge g, int prec) { return prec == HISQ_F64 ? 18 : g->recon_U; }
 int link_recon_n(hisq_gauge g, int prec) { return prec == HISQ_F64 ? 18 : g->recon_N; }
 
-// rhs per thread of the fixed-point FP64 kernel: two share the link loads once
-// the threads fill the SMs one and a half times over at 12 warps each (48^3x12,
-// n = 8: 1.89 ms against 2.06 with one), else one, for more warps in flight
-// (16^4, n = 4: 58 us against 66).
-int auto_rpt_fx64(hisq_gauge g, int n) {
-    return n % 2 == 0 && (long long)g->g.vh * (n / 2) >= 18ll * 32 * device_sm_count() ? 2 : n > 8 ? 2 : 1;
-}
+// rhs per thread of the fixed-point FP64 kernel: one, and two beyond the eight
+// groups of a block (see dslash_fx64.cuh for the times).
+int auto_rpt_fx64(int n) { return n > 8 ? 2 : 1; }
 
 int auto_rpt(int n, int prec) {
     const int mx = dslash_max_rpt(prec);
@@ -573,7 +569,7 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
     }
     int r = requested ? requested : g->tune_rpt;
     if (r == 0 || r > dslash_max_rpt(prec) || n % r != 0 || n / r > 8)
-        r = prec == HISQ_F64 && g->fx ? auto_rpt_fx64(g, n) : auto_rpt(n, prec);
+        r = prec == HISQ_F64 && g->fx ? auto_rpt_fx64(n) : auto_rpt(n, prec);
     DslashTune t = dslash_default_tune(prec, r, layout);
     const int kind = kind_of_flags(g->tune_flags);
     if (!requested && g->tune_minb && r == g->tune_rpt && dslash_mapping_built(prec, r, g->tune_minb, kind) &&

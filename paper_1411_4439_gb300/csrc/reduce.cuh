@@ -111,7 +111,7 @@ struct FinState {
     double rr, rr_rel, freeze2, alpha_max;
 };
 __device__ __forceinline__ FinState fin_load(const CgScalars* cg, int k) {
-    FinState f;
+    FinState f = {};
     if (cg == nullptr) return f;
     const int act = cg->active[k], frz = cg->frozen[k];
     f.stall = cg->stall[k];
