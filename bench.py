@@ -187,10 +187,10 @@ class ClockSampler:
 # capture of that kernel (profiles/), keyed by (precision, lattice, n, rhs per
 # thread, min blocks, mapping flags). A mapping without a capture reports null.
 DSLASH_TRAFFIC = {
-    # profiles/dslash_bundle_f16_r18_r14_n8_48x48x48x12.md: 418.9 MB read + 37.1 MB written
-    ("f16", (48, 48, 48, 12), 8, 8, 4, 132): 455975424,
-    # profiles/dslash_bundle_f32_r18_r14_n8_48x48x48x12.md: 831.5 MB read + 100.1 MB written
-    ("f32", (48, 48, 48, 12), 8, 8, 3, 0): 931567104,
+    # profiles/dslash_bundle_f16_r18_r14_n8_48x48x48x12.md: 411.8 MB read + 54.6 MB written
+    ("f16", (48, 48, 48, 12), 8, 8, 4, 132): 466410496,
+    # profiles/dslash_bundle_f32_r18_r14_n8_48x48x48x12.md: 824.4 MB read + 99.5 MB written
+    ("f32", (48, 48, 48, 12), 8, 8, 3, 0): 923935488,
 }
 
 
@@ -338,13 +338,14 @@ def run_gpu(args):
         e1.record(stream)
         e1.synchronize()
         durs.append(e0.elapsed_time(e1) / 1e3)
-        # per iteration: two Dslash, update_r, update_px; per reliable update:
-        # accumulate, two FP64 Dslash, best-iterate copy, rescale; per solve:
+        # per iteration: two Dslash and the sums over the second one's blocks,
+        # update_r, update_px; per reliable update: accumulate, two FP64 Dslash
+        # and the sums, best-iterate copy, rescale; per solve:
         # norm |b|, copy the residual, best-iterate copy, rescale; per chunk
         # of check_every iterations of the device-driven loop: the decision
         # and booking kernels
         chunks = -(-st.total_iters // params.check_every)
-        launches += 4 * st.total_iters + 5 * st.reliable_updates + 4 + 2 * chunks
+        launches += 5 * st.total_iters + 6 * st.reliable_updates + 4 + 2 * chunks
         stats_last = st
     torch.cuda.synchronize(dev)
     wall = time.perf_counter() - wall0
