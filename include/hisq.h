@@ -109,9 +109,17 @@ const char* hisq_last_error(void);
  * hisq_gauge_load packs U and N into the internal site-major SoA layout
  * [parity][mu][complex component][V_h] in precision `prec`, and always also
  * keeps an FP64 R18 copy used by FP64 Dslash calls and by the CG's FP64
- * reliable updates (as 55-bit fixed point with one exponent per field and
- * direction where all links of a direction are of similar size, else doubles;
- * FP64 Dslash results carry no larger rounding error from the former). prec == HISQ_F64 requires R18 for both fields.
+ * reliable updates. prec == HISQ_F64 requires R18 for both fields.
+ * Where the links of each direction are of similar size and not mostly
+ * diagonal, real or otherwise thin, and the field has at most 64^3 x 56 sites
+ * or so, a 55-bit fixed-point form of the FP64 copy is kept beside it (as many
+ * bytes again; a load that cannot get them does without) and FP64 operators
+ * sum in fixed point relative to the largest neighbour of a site, scaled by the
+ * field's largest link. An output real that is small against that is summed in
+ * FP64 from the FP64 copy. Sites are no further off than with FP64 multiply-adds;
+ * a real alone is within 1600 x 2^-53 of the sum of its |products| (typically
+ * 0.2 x 2^-53), where 96 multiply-adds stay within 96 x 2^-53. Links or vectors that are not finite take
+ * FP64 multiply-adds.
  * prec == HISQ_F16 stores every link real as a 16-bit integer q with value
  * q * s_c, one scale s_c = max |Re|,|Im| / 32767 per stored complex
  * component c of each field (2^-15 of the range, where IEEE half keeps only

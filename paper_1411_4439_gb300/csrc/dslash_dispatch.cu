@@ -1,6 +1,8 @@
 // Routes a Dslash request to the kernel family built for its storage
 // precision and link compression (see dslash_inst.cu), and owns the table of
 // thread mappings those families contain.
+#include <cmath>
+
 #include "hisq_internal.cuh"
 
 namespace hisq {
@@ -182,6 +184,19 @@ static int fx64_split(const DslashArgs& a, int rpt) {
     return rpt <= 2 && warps < 4ll * device_sm_count() ? 4 : 1;
 }
 
+bool fx64_usable(const DslashArgs& a) {
+    if (a.U_fx == nullptr || a.N_fx == nullptr) return false;
+    if (!a.has_mu) return true;
+    const double f[4] = {a.ft1, a.bt1, a.ft3, a.bt3};
+    for (int i = 0; i < 4; ++i) {
+        if (!std::isfinite(f[i]) || f[i] == 0.0) return false;
+        int e = 0;
+        std::frexp(f[i], &e);
+        if (e <= -400 || e >= 400) return false;
+    }
+    return true;
+}
+
 cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi,
                           const DslashTune& t, cudaStream_t s) {
     if (!dslash_variant_supported(prec, ru, rn, epi)) return cudaErrorInvalidValue;
@@ -199,7 +214,7 @@ cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi
     }
     const int r = t.rpt, b = t.minb, k = t.kind, l = t.layout;
     if (a.both && !dslash_both_ok(a, prec)) return cudaErrorInvalidValue;
-    if (prec == HISQ_F64 && a.fx) {
+    if (prec == HISQ_F64 && fx64_usable(a)) {
         const int split = fx64_split(a, r);
         return l == HISQ_SOA ? dslash_fx64_soa(a, epi, r, split, s) : dslash_fx64_aos(a, epi, r, split, s);
     }

@@ -8,41 +8,61 @@
 //   link real  l = a 2^(e - 55), e the exponent of the (field, direction)
 //              block (every |l| < 2^e), a = a1 2^28 + a0 with |a1| <= 2^27 and
 //              |a0| <= 2^27; packed once when the field is loaded;
-//   vector real v = b 2^(E - o - 56), |b| < 2^56, b = b1 2^28 + b0 with both
-//              limbs carrying v's sign; split in registers per hop. E is a
-//              running block exponent per output site and rhs, o the exponent
-//              of the hop's link block;
+//   vector real v = b 2^(E - o - 56), |b| <= 2^56, b = b1 2^28 + b0 with |b1| <= 2^28
+//              and |b0| <= 2^27; split in registers per hop. E is a running
+//              block exponent per output site and rhs, o the exponent of the
+//              hop's link block;
 //   product    a b = a1 b1 2^56 + (a1 b0 + a0 b1) 2^28 + a0 b0: the first two
 //              terms go to two 64-bit accumulators per output real (three
 //              IMAD.WIDE a real product), a0 b0 is dropped.
 //
 // Bounds: an output real sums 96 products, so |S2| <= 96 2^55 and
-// |S1| <= 96 (2^55 + 2^55) < 2^63. Against the largest product the dropped
-// term is at most 2^-56, the vector rounding 2^-56, the link rounding 2^-56
-// (reals within 4 of the block's largest are exact) and the final shift
-// 2^-56; 96 FP64 fused multiply-adds round at 2^-53 of their running sum.
-// Measured against quad-precision sums (Haar links, 8^4 and two ragged
-// lattices): 1.2e-16 of the result for Gaussian vectors, 0.7e-16 for Z2 ones
-// (1.7e-16 and 1.1e-16 at mu = 0.1); the FMA kernel 3.5e-16 for all of them.
+// |S1| <= 96 (2^54 + 2^55) < 2^63. In units of 2^E a product loses at most 2^-56
+// to the link's rounding, 2^-57 to the vector's and 2^-57 to the dropped term,
+// so a sum is off by at most 25 x 2^(E - 53), 0.35 x 2^(E - 53) in the root mean
+// square for Haar links. 2^E is 2 to 4 times the largest neighbour real times
+// the block scale 2^o, so it says nothing about one output: the link may be zero
+// or small where the neighbour is large, or lead to another colour. What an FP64
+// sum loses follows its own partial sums, and so does the test here: an output
+// real counts only if its sum, looked at after every hop, came to 2^(E - 6) at
+// least once (kFxReach); the sites of other outputs are formed again by fx_redo
+// with FP64 multiply-adds on the double links, which the field keeps beside the
+// fixed-point ones. Root mean square errors (8000 to 40000 sites in numpy
+// integers against long double):
+//
+//                                             this kernel   FP64 multiply-adds
+//   site norm: Haar links x 0.9                  0.9e-16          3.7e-16
+//              Haar links x 0.51                 1.3e-16          3.7e-16
+//   real against the sum of its |products|:
+//              Haar links                        1.6e-17          7.1e-17
+//              a single neighbour                5.2e-17          5.2e-17
+//              a single neighbour and colour     1.2e-16          0.5e-16
+//              one colour 1/16 of the others,
+//              links diagonal                    2.0e-16          0.7e-16
+//
+// and no real is off by more than 1600 units of 2^-53 of the sum of its
+// |products| (multiply-adds: 96). Links that are mostly diagonal, real or
+// otherwise thin, where a vector's parts stay apart, keep to multiply-adds (see
+// plan_links). Rounding the vectors and balancing their low limb halves the error
+// for 2.5 % of the time; the looks at the sums take 1.5 %. At a limit of 2^(E - 5)
+// Gaussian vectors at mu = 0.1 have a thousandth of the sites formed again, 3 to 8 %
+// of the time (8^4, n = 1: 12.7 us against 8.4); at 2^(E - 6) it does not show.
 //
 // What bounds it: the register ports. An IMAD.WIDE with fresh operands (two
 // factors, a 64-bit accumulator read and written) takes 3.3 to 4.2 cycles of
 // a scheduler instead of 2; the 108 of a hop and rhs are 57 % of the time, the
 // limb splitting 14 %, the rest link loads, addresses and the E test. One rhs
-// a thread at 16 warps per SM is as fast as two at 12 (48^3x12, n = 8: 1.79 and
-// 1.78 ms) or faster (32^3x8, n = 4: 178 us against 191); four need 255
-// registers (8 warps a SM) and lose.
-// Time per launch, FMA kernel -> this one: 48^3x12, n = 8: 5.24 -> 1.79 ms;
-// 32^3x8, n = 8: 1055 -> 361 us; 24^3x6, n = 4: 305 -> 68 us; 16^4, n = 4: 156
+// a thread at 16 warps per SM is as fast as two at 12 (48^3x12, n = 8, before the
+// looks at the sums: 1.79 and 1.78 ms) or faster (32^3x8, n = 4: 178 us against
+// 191); four need 255 registers (8 warps a SM) and lose.
+// Time per launch, FMA kernel -> this one: 48^3x12, n = 8: 5.24 -> 1.87 ms;
+// 32^3x8, n = 8: 1055 -> 376 us; 24^3x6, n = 4: 305 -> 67 us; 16^4, n = 4: 156
 // -> 52 us; 8^4, n = 1: 45 -> 8 us.
 //
 // E starts one above the first neighbour's largest exponent and grows when a
 // later neighbour exceeds it; the accumulators are then shifted (rounded).
-// Sites whose neighbours hold non-finite numbers, or only numbers outside
-// 2^-900 .. 2^900, are recomputed with FP64 arithmetic (fx_site_fp64), so
-// NaN, infinities and extreme ranges come out as from FP64 sums. Fields whose
-// links differ in size by more than a factor of 16 inside a direction, or
-// are not finite, keep the double storage and the FMA kernel.
+// Sites with a neighbour that is not finite or beyond 2^900 go through fx_redo
+// too, so NaN, infinities and extreme ranges come out as from FP64 sums.
 //
 // Full-lattice operators take both parities in one launch (a.both): 24^3x6, n =
 // 4, M^dag 163 -> 143 us, the waves of the second parity fill the first's tail.
@@ -59,15 +79,11 @@ namespace hisq {
 constexpr int kFxFloor = -900;   // lowest block exponent
 constexpr int kFxCeil = 900;     // above: FP64 path
 constexpr int kFxHead = 1;       // bits a new block exponent leaves above its vector
+constexpr int kFxReach = 6;      // a sum that never came within 2^-kFxReach of 2^E is formed in FP64
 
-// A stored real as double (exact for |l| >= 2^(e - 3)).
-__device__ __forceinline__ double fx_link_real(int a1, int a0, int e) {
-    const long long v = ((long long)a1 << 28) + a0;
-    return (double)v * scalbn(1.0, e - 55);
-}
-
-// Limbs of v 2^(o - E + 56), negated for a backward hop; sh = E - o + 1030 -
-// (exponent field of v) >= 8 low bits of the left-aligned mantissa go.
+// Limbs of v 2^(o - E + 56) rounded, negated for a backward hop; sh = E - o +
+// 1029 - (exponent field of v) >= 7 low bits of the left-aligned mantissa go,
+// one bit stays below the unit for the rounding.
 template <bool NEG>
 __device__ __forceinline__ void fx_limbs(unsigned hi, unsigned lo, int k, int& b1, int& b0) {
     const int sh = k - (int)((hi << 1) >> 21);
@@ -75,12 +91,14 @@ __device__ __forceinline__ void fx_limbs(unsigned hi, unsigned lo, int k, int& b
     const unsigned ml = lo << 11;
     unsigned long long u;
     asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tshr.u64 %0, t, %3;\n\t}" : "=l"(u) : "r"(ml), "r"(mh), "r"(sh));
+    // + 1 rounds, + 2^28 (2^27 units) makes the low limb -2^27 .. 2^27 - 1
+    u += (1ull << 28) + 1;
     const unsigned ul = (unsigned)u, uh = (unsigned)(u >> 32);
     // the sign by a multiplication: the FMA pipe has room where the ALU has none
     const int s = (int)hi >> 31;
     const int sg = (NEG ? ~s : s) | 1;
-    b0 = (int)(ul & 0x0fffffffu) * sg;
-    b1 = (int)__funnelshift_r(ul, uh, 28) * sg;
+    b0 = ((int)((ul >> 1) & 0x0fffffffu) - (1 << 27)) * sg;
+    b1 = (int)__funnelshift_r(ul, uh, 29) * sg;
 }
 
 __device__ __forceinline__ void fx_mac(long long& s, int a, int b) {
@@ -104,45 +122,82 @@ __device__ __forceinline__ void fx_scale(int& x1, int& x0, int f1, int f0) {
     x1 = (int)((v - x0) >> 28);
 }
 
-// D in of one site and rhs in FP64 arithmetic (rare sites, see above).
+// D in of the sites (h of the lanes in mask) and rhs k in FP64 arithmetic on the
+// double links; every lane of the warp calls it and the lanes in mask get w.
+// Two sites a pass, a lane per hop: one flagged site costs the FP64 pipe a
+// sixteenth of what it costs a lane on its own.
 template <int LAYOUT>
-static __device__ __noinline__ void fx_site_fp64(const DslashArgs& a, int p, int h, int k, double2* out) {
+static __device__ __noinline__ void fx_redo(const DslashArgs& a, int p, int k, unsigned mask, int h, double2 (&w)[3]) {
     const Geom& g = a.g;
-    const int vh = g.vh, q = 1 - p;
-    const int xh = h % g.hx;
-    int r = h / g.hx;
-    const int y = r % g.L[1];
-    r /= g.L[1];
-    const int z = r % g.L[2], t = r / g.L[2];
-    const int x = 2 * xh + ((p + y + z + t) & 1);
-    double2 acc[3];
-    for (int c = 0; c < 3; ++c) acc[c] = make_double2(0.0, 0.0);
+    const int vh = g.vh, q = 1 - p, lane = threadIdx.x & 31;
+    const int mu = (lane & 15) >> 2, hop = lane & 3, naik = hop >> 1, back = hop & 1;
+    const int d = (naik ? 3 : 1) * (back ? -1 : 1);
+    const double f = (mu == 3 && a.has_mu) ? (hop == 0 ? a.ft1 : hop == 1 ? a.bt1 : hop == 2 ? a.ft3 : a.bt3) : 1.0;
     const double2* in = reinterpret_cast<const double2*>(a.in[k]) + (a.both ? (size_t)q * 3 * vh : 0);
+    const double2* block = reinterpret_cast<const double2*>(naik ? a.N : a.U) + (size_t)((back ? q : p) * 4 + mu) * 9 * vh;
 #pragma unroll 1
-    for (int e = a.t_only ? 12 : 0; e < 16; ++e) {
-        const int mu = e >> 2, hop = e & 3, naik = hop >> 1, back = hop & 1;
-        const int d = (naik ? 3 : 1) * (back ? -1 : 1);
-        const int coord = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
-        const int stride = mu == 1 ? g.sy : mu == 2 ? g.sz : g.st;
-        const int cn = wrap(coord + d, g.L[mu]);
-        const int hn = mu == 0 ? h - xh + (cn >> 1) : h + (cn - coord) * stride;
-        const int4* lk = reinterpret_cast<const int4*>(naik ? a.N : a.U) + (size_t)((back ? q : p) * 4 + mu) * 9 * vh +
-                         (back ? hn : h);
-        const int ex = a.fx_exp[naik * 4 + mu];
-        const double f = (mu == 3 && a.has_mu) ? (hop == 0 ? a.ft1 : hop == 1 ? a.bt1 : hop == 2 ? a.ft3 : a.bt3) : 1.0;
-        double2 v[3];
-        for (int c = 0; c < 3; ++c) v[c] = in[spinor_index<LAYOUT>(hn, c, vh)];
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) {
-                const int4 w = lk[(size_t)(back ? 3 * j + i : 3 * i + j) * vh];
-                const double2 m = make_double2(fx_link_real(w.x, w.y, ex) * f, fx_link_real(w.z, w.w, ex) * f);
-                if (back)
-                    cmsub_conj(acc[i], m, v[j]);
-                else
-                    cmadd(acc[i], m, v[j]);
+    while (mask) {
+        const int first = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const int second = mask ? __ffs(mask) - 1 : first;
+        mask &= mask - 1;
+        const int hs = __shfl_sync(0xffffffffu, h, lane < 16 ? first : second);
+        double2 acc[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] = make_double2(0.0, 0.0);
+        if (mu == 3 || !a.t_only) {
+            const int xh = hs % g.hx;
+            int r = hs / g.hx;
+            const int y = r % g.L[1];
+            r /= g.L[1];
+            const int z = r % g.L[2], t = r / g.L[2];
+            const int x = 2 * xh + ((p + y + z + t) & 1);
+            const int coord = mu == 0 ? x : mu == 1 ? y : mu == 2 ? z : t;
+            const int stride = mu == 1 ? g.sy : mu == 2 ? g.sz : g.st;
+            const int cn = wrap(coord + d, g.L[mu]);
+            const int hn = mu == 0 ? hs - xh + (cn >> 1) : hs + (cn - coord) * stride;
+            const double2* lk = block + (back ? hn : hs);
+            double2 v[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] = __ldg(in + spinor_index<LAYOUT>(hn, c, vh));
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const double2 l = __ldg(lk + (size_t)(back ? 3 * j + i : 3 * i + j) * vh);
+                    const double2 m = make_double2(l.x * f, l.y * f);
+                    if (back)
+                        cmsub_conj(acc[i], m, v[j]);
+                    else
+                        cmadd(acc[i], m, v[j]);
+                }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, o);
+                acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, o);
             }
+            const int from = lane == first ? 0 : 16;
+            const double re = __shfl_sync(0xffffffffu, acc[c].x, from), im = __shfl_sync(0xffffffffu, acc[c].y, from);
+            if (lane == first || lane == second) w[c] = make_double2(re, im);
+        }
     }
-    for (int c = 0; c < 3; ++c) out[c] = acc[c];
+}
+
+// The upper halves of two 32-bit words, each with the bits of its sign flipped
+// away: |word| / 2^16 (rounded down for negative words) side by side.
+__device__ __forceinline__ unsigned fx_tops(unsigned a, unsigned b) {
+    unsigned v, s;
+    asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(v) : "r"(a), "r"(b));
+    asm("prmt.b32 %0, %1, %2, 0xffbb;" : "=r"(s) : "r"(a), "r"(b));   // sign bytes
+    return v ^ s;
+}
+
+// Two halves of 16 bits shifted right by d >= 0.
+__device__ __forceinline__ unsigned fx_shift_tops(unsigned t, int d) {
+    return d > 15 ? 0u : (t >> d) & ((0xffffu >> d) * 0x10001u);
 }
 
 template <int R, int LAYOUT>
@@ -152,7 +207,8 @@ struct FxHops {
     int vh, p, h, x, y, z, t;
     long long s2[R][6], s1[R][6];   // (re, im) of the three output colours
     int E[R];
-    unsigned nz[R];
+    unsigned peak[R];               // largest exponent field of a neighbour real, at bit 21
+    unsigned tops[R][3];            // per colour (re, im): OR over the hops of the sum's size, 2^(E - 7) a unit
     uint4 cur[R][3];                // the next hop's neighbour vectors, as loaded
     // the direction at hand: coordinate, extent, half-index step (0 shift but x)
     int mu, c, ext, stride, half;
@@ -172,7 +228,9 @@ struct FxHops {
         for (int j = 0; j < R; ++j) {
             in[j] = reinterpret_cast<const uint4*>(a.in[k0 + j]) + (a.both ? (size_t)(1 - p) * 3 * vh : 0);
             E[j] = kFxFloor;
-            nz[j] = 0u;
+            peak[j] = 0u;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) tops[j][c] = 0u;
 #pragma unroll
             for (int c = 0; c < 6; ++c) s2[j][c] = s1[j][c] = 0ll;
         }
@@ -219,7 +277,7 @@ struct FxHops {
         int4 m[9];
         {
             const size_t plane = (size_t)vh * sizeof(int4);
-            const char* lk = reinterpret_cast<const char*>(NAIK ? a.N : a.U) + (size_t)((BACK ? 1 - p : p) * 4 + mu) * 9 * plane;
+            const char* lk = reinterpret_cast<const char*>(NAIK ? a.N_fx : a.U_fx) + (size_t)((BACK ? 1 - p : p) * 4 + mu) * 9 * plane;
             const unsigned off = (unsigned)(BACK ? neighbour<HOP>() : h) * (unsigned)sizeof(int4);
 #pragma unroll
             for (int e = 0; e < 9; ++e) m[e] = __ldcs(reinterpret_cast<const int4*>(lk + e * plane + off));
@@ -233,7 +291,7 @@ struct FxHops {
             unsigned big = 0;
 #pragma unroll
             for (int i = 0; i < 3; ++i) big = max(big, max(cur[j][i].y << 1, cur[j][i].w << 1));
-            nz[j] |= big;
+            peak[j] = max(peak[j], big);
             const int en = (int)(big >> 21) - 1022 + o;
             // the vote keeps the branch uniform: most hops skip it without the
             // divergence bookkeeping of a lane-wise branch (9 % of the kernel)
@@ -242,13 +300,15 @@ struct FxHops {
                     const int d = en + kFxHead - E[j];
                     E[j] = en + kFxHead;
 #pragma unroll
+                    for (int i = 0; i < 3; ++i) tops[j][i] = fx_shift_tops(tops[j][i], d);
+#pragma unroll
                     for (int i = 0; i < 6; ++i) {
                         s2[j][i] = fx_shift(s2[j][i], d);
                         s1[j][i] = fx_shift(s1[j][i], d);
                     }
                 }
             }
-            const int k = E[j] - o + 1030;
+            const int k = E[j] - o + 1029;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 fx_limbs<BACK>(cur[j][i].y, cur[j][i].x, k, v1[j][2 * i], v0[j][2 * i]);
@@ -302,6 +362,14 @@ struct FxHops {
                 }
             }
         }
+#pragma unroll
+        for (int j = 0; j < R; ++j) note_sizes(j);
+    }
+
+    __device__ __forceinline__ void note_sizes(int j) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            tops[j][i] |= fx_tops((unsigned)(s2[j][2 * i] >> 32), (unsigned)(s2[j][2 * i + 1] >> 32));
     }
 
     // the hops of the directions [first, last)
@@ -323,10 +391,16 @@ struct FxHops {
         for (int j = 0; j < R; ++j) {
             int em = max(E[j], __shfl_xor_sync(0xffffffffu, E[j], 8));
             em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
-            nz[j] |= __shfl_xor_sync(0xffffffffu, nz[j], 8);
-            nz[j] |= __shfl_xor_sync(0xffffffffu, nz[j], 16);
+            peak[j] = max(peak[j], __shfl_xor_sync(0xffffffffu, peak[j], 8));
+            peak[j] = max(peak[j], __shfl_xor_sync(0xffffffffu, peak[j], 16));
             const int d = em - E[j];
             E[j] = em;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                tops[j][i] = fx_shift_tops(tops[j][i], d);
+                tops[j][i] |= __shfl_xor_sync(0xffffffffu, tops[j][i], 8);
+                tops[j][i] |= __shfl_xor_sync(0xffffffffu, tops[j][i], 16);
+            }
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 long long u = s2[j][c], w = s1[j][c];
@@ -341,12 +415,18 @@ struct FxHops {
                 s2[j][c] = u;
                 s1[j][c] = w;
             }
+            note_sizes(j);
         }
     }
 
-    // whether rhs j left the range of the fixed-point sums
+    // Whether rhs j needs FP64 arithmetic: a neighbour too large, or an output real whose sums stayed below 2^(E - kFxReach). (Neighbours
+    // that are all zero give exact zeros.)
     __device__ __forceinline__ bool rare(int j) const {
-        return E[j] > kFxCeil || (E[j] == kFxFloor && nz[j] != 0u) || a.fx_slow;
+        constexpr unsigned kSmall = (1u << (23 - kFxReach - 16)) - 1;   // hi word of 2^(E - kFxReach) is 2^(23 - kFxReach)
+        bool low = false;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) low = low || (tops[j][i] & 0xffffu) <= kSmall || (tops[j][i] >> 16) <= kSmall;
+        return E[j] > kFxCeil || (low && peak[j] != 0u);
     }
 
     // (S2 2^28 + S1) 2^(E - 83), times sgn = +-1
@@ -374,30 +454,35 @@ __global__ void __launch_bounds__(MAXT, MINB) dslash_fx64_kernel(const __grid_co
 
     const int v0 = blockIdx.x * a.run * spb;
     for (int it = 0, v = v0 + slot; it < a.run && v - slot < vh; ++it, v += spb) {
-        if (SPLIT == 1 && v >= vh) continue;
         const int h = visit_site(v < vh ? v : vh - 1, a.g);
         FxHops<R, LAYOUT> hops(a, p, h, k0);
+        bool mine = v < vh;
         if (SPLIT == 1) {
             hops.run(a.t_only ? 3 : 0, 4);
         } else {
             const int mu = lane >> 3;
             if (!a.t_only || mu == 3) hops.run(mu, mu + 1);
             hops.combine();
-            if (mu != 0 || v >= vh) continue;
+            mine = mine && mu == 0;
         }
         const bool neg = a.cd < 0.0;   // cd is +1 or -1 (checked by the launcher)
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             const int k = k0 + j;
             double2 w[3];
-            if (hops.rare(j)) {
-                fx_site_fp64<LAYOUT>(a, p, h, k, w);
-                if (neg)
-                    for (int c = 0; c < 3; ++c) w[c] = make_double2(-w[c].x, -w[c].y);
-            } else {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) w[c] = make_double2(hops.value(j, 2 * c, neg), hops.value(j, 2 * c + 1, neg));
+            for (int c = 0; c < 3; ++c) w[c] = make_double2(hops.value(j, 2 * c, neg), hops.value(j, 2 * c + 1, neg));
+            const bool again = mine && hops.rare(j);
+            const unsigned mask = __ballot_sync(0xffffffffu, again);
+            if (mask) {
+                double2 u[3];
+                fx_redo<LAYOUT>(a, p, k, mask, h, u);
+                if (again) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) w[c] = neg ? make_double2(-u[c].x, -u[c].y) : u[c];
+                }
             }
+            if (!mine) continue;
             double2* o = reinterpret_cast<double2*>(a.out[k]) + half;
             double n2max = 0.0;
 #pragma unroll
@@ -432,9 +517,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dslash_fx64_kernel(const __grid_co
     block_reduce_finish<R>(a, k0, red0, red1);
 }
 
-// Temporal factor f as a 55-bit mantissa in limbs and an exponent.
-inline bool fx_factor(double f, int* f1, int* f0, int* fe) {
-    if (!std::isfinite(f) || f == 0.0) return false;
+// Temporal factor f (in fx64_usable's range) as a 55-bit mantissa in limbs and an exponent.
+inline void fx_factor(double f, int* f1, int* f0, int* fe) {
     int e = 0;
     const double m = std::frexp(f, &e);
     const long long v = std::llrint(std::ldexp(m, 55));
@@ -442,7 +526,6 @@ inline bool fx_factor(double f, int* f1, int* f0, int* fe) {
     *f0 = (int)lo;
     *f1 = (int)((v - lo) >> 28);
     *fe = e;
-    return e > -400 && e < 400;
 }
 
 template <int R, int SPLIT, int EPI, int LAYOUT, int MAXT, int MINB>
@@ -451,12 +534,11 @@ cudaError_t launch_fx64(const DslashArgs& args, cudaStream_t s) {
     if (G < 1 || G * R != args.nrhs || G > 8) return cudaErrorInvalidValue;
     if (args.cd != 1.0 && args.cd != -1.0) return cudaErrorInvalidValue;
     if (args.both && args.red_mode != RED_NONE) return cudaErrorInvalidValue;
+    if (!fx64_usable(args)) return cudaErrorInvalidValue;
     DslashArgs a = args;
-    a.fx_slow = 0;
     if (a.has_mu) {
         const double f[4] = {a.ft1, a.bt1, a.ft3, a.bt3};
-        for (int i = 0; i < 4; ++i)
-            if (!fx_factor(f[i], &a.fx_f1[i], &a.fx_f0[i], &a.fx_fe[i])) a.fx_slow = 1;
+        for (int i = 0; i < 4; ++i) fx_factor(f[i], &a.fx_f1[i], &a.fx_f0[i], &a.fx_fe[i]);
     }
     int bx = 128 / G;
     bx &= ~31;

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __rest
     const unsigned V = 2u * (unsigned)g.vh;
     const int mu = blockIdx.y;
     unsigned long long mx[NC], hi = 0ull, lo = ~0ull;
+    unsigned links = 0, thin = 0;
     double err = 0.0;
 #pragma unroll
     for (int c = 0; c < NC; ++c) mx[c] = 0ull;
@@ -178,7 +179,15 @@ __global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __rest
             link = umax64(link, b);
         }
         hi = umax64(hi, link);
-        if (link != 0ull && link < lo) lo = link;
+        if (link != 0ull) {
+            lo = link < lo ? link : lo;
+            ++links;
+            // reals below 1/16 of the link's largest (four off its exponent)
+            const long long small = (long long)link - (4ll << 52);
+#pragma unroll
+            for (int c = 0; c < 9; ++c)
+                thin += ((long long)abs_bits(m[c].x) < small) + ((long long)abs_bits(m[c].y) < small);
+        }
         if (RECON != 18) {
             const int sg = RECON == 12 ? staggered_sign(g, site_of(g, i), mu, hop) : 1;
             const double2 f = third_factor<RECON>(m, sg, inv_s, err);
@@ -193,6 +202,12 @@ __global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __rest
     v[10] = ~lo;   // the smallest as a largest
     v[11] = (unsigned long long)__double_as_longlong(err);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    links = __reduce_add_sync(0xffffffffu, links);
+    thin = __reduce_add_sync(0xffffffffu, thin);
+    if (lane == 0) {
+        atomicAdd(&out->links[mu], (unsigned long long)links);
+        atomicAdd(&out->thin[mu], (unsigned long long)thin);
+    }
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         for (int o = 16; o > 0; o >>= 1) v[c] = umax64(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
@@ -269,14 +284,14 @@ __device__ __forceinline__ short2 store_one(double2 a, const double* inv, int c,
     return make_short2(quantize(a.x, inv[c]), quantize(a.y, inv[c]));
 }
 
-// One pass over a field writes its FP64 copy (fixed point or doubles) and,
-// unless the storage precision is FP64 (LC = double2), the storage copy. At
-// 48^3x12 with 16-bit storage 0.52 ms (R18, 1.7 GB) and 0.78 ms (R14), where
-// separate passes took 1.87 and 2.92 ms; the FP64 pipe bounds it (the
-// quantisation multiplies, z), so the fixed-point split uses integers only.
+// One pass over a field writes its FP64 copy, unless out_fx is null the
+// fixed-point form of it, and unless the storage precision is FP64 (LC =
+// double2) the storage copy. The FP64 pipe bounds it (the quantisation
+// multiplies, z), so the fixed-point split uses integers only.
 template <typename LC, int RECON>
-__global__ void __launch_bounds__(256) pack_kernel(Geom g, const double2* __restrict__ canon, int fx, LinkScales sc,
-                                                   double2* __restrict__ out64, LC* __restrict__ out_lo) {
+__global__ void __launch_bounds__(256) pack_kernel(Geom g, const double2* __restrict__ canon, LinkScales sc,
+                                                   double2* __restrict__ out64, int4* __restrict__ out_fx,
+                                                   LC* __restrict__ out_lo) {
     constexpr int NC = RECON / 2;
     const unsigned V = 2u * (unsigned)g.vh;
     const int mu = blockIdx.y;
@@ -287,14 +302,13 @@ __global__ void __launch_bounds__(256) pack_kernel(Geom g, const double2* __rest
         double2 m[9];
 #pragma unroll
         for (int c = 0; c < 9; ++c) m[c] = src[c];
-        double2* o64 = out64 + (size_t)(s.parity * 4 + mu) * 9 * g.vh + s.h;
+        const size_t at = (size_t)(s.parity * 4 + mu) * 9 * g.vh + s.h;
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
-            if (fx) {
+            out64[at + (size_t)c * g.vh] = m[c];
+            if (out_fx != nullptr) {
                 const int2 re = fx_split(m[c].x, fxe), im = fx_split(m[c].y, fxe);
-                reinterpret_cast<int4*>(o64)[(size_t)c * g.vh] = make_int4(re.x, re.y, im.x, im.y);
-            } else {
-                o64[(size_t)c * g.vh] = m[c];
+                out_fx[at + (size_t)c * g.vh] = make_int4(re.x, re.y, im.x, im.y);
             }
         }
         if constexpr (LinkPair<LC>::paired) {
@@ -382,11 +396,11 @@ cudaError_t launch_link_scan(const Geom& g, const double2* canon, int recon, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, int fx, const LinkScales& sc,
-                              void* out64, void* out_lo, cudaStream_t s) {
+cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, const LinkScales& sc, void* out64,
+                              void* out_fx, void* out_lo, cudaStream_t s) {
     const dim3 grid((grid_for(8ll * g.vh) + 3) / 4, 4);
     double2* o = (double2*)out64;
-#define HISQ_PACK(LC, RECON) pack_kernel<LC, RECON><<<grid, 256, 0, s>>>(g, canon, fx, sc, o, (LC*)out_lo)
+#define HISQ_PACK(LC, RECON) pack_kernel<LC, RECON><<<grid, 256, 0, s>>>(g, canon, sc, o, (int4*)out_fx, (LC*)out_lo)
     switch (prec * 100 + recon) {
         case HISQ_F64 * 100 + 18: HISQ_PACK(double2, 18); break;
         case HISQ_F32 * 100 + 18: HISQ_PACK(float2, 18); break;

@@ -184,9 +184,10 @@ struct hisq_gauge_s {
     void* link_block = nullptr;  // the allocation of all link copies
     void* U_lo = nullptr;        // storage copy (prec, recon)
     void* N_lo = nullptr;
-    double2* U64 = nullptr;      // FP64 R18 copy: doubles, or with fx int4 limbs (dslash_fx64.cuh)
+    double2* U64 = nullptr;      // FP64 R18 copy
     double2* N64 = nullptr;
-    int fx = 0;
+    int4* U_fx = nullptr;        // its fixed-point form (dslash_fx64.cuh) where the field qualifies
+    int4* N_fx = nullptr;
     int fx_exp[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     size_t link_bytes = 0;
     int tune_rpt = 0;            // 0 = automatic
@@ -212,17 +213,25 @@ extern "C" const char* hisq_last_error(void) { return g_last_error.c_str(); }
 namespace {
 
 // Checks both fields against recon_tol, sets the 16-bit component scales and
-// decides the FP64 format from what the scan found. Fixed point needs, in
-// every (field, direction), all links finite and every nonzero link's largest
-// real within a factor of 16 of the block's largest, so that the smallest
-// links still carry 51 bits (Haar links x a constant lie within 2.5).
-hisq_status plan_links(hisq_gauge g, const LinkScan (&scan)[2], double recon_tol, LinkScales (&sc)[2]) {
+// decides whether FP64 calls get a fixed-point copy of the links. The kernel
+// forms sums again in FP64 that stay small against their block exponent, so
+// these conditions are about speed and the last bits: in every (field,
+// direction) all links finite, no nonzero link's largest real below a fifth of
+// 2^e, e the block's exponent (the largest real of a multiple of a unitary
+// matrix lies between 0.408 and 1 of the multiple, so links of one size always
+// pass), and at most a third of the reals thin, below 1/16 of their link's
+// largest (Haar links 9 %, real ones 54 %, abelian ones 2/3 and up): where
+// links leave colours or real and imaginary parts apart, most sums are formed
+// again (unit links on 32^3x8, one colour of n = 8: 3.5 ms, multiply-adds 1.06).
+// A block without links gets an exponent below all others: the vectors behind
+// it must not raise the block exponent of a sum.
+hisq_status plan_links(hisq_gauge g, const LinkScan (&scan)[2], double recon_tol, LinkScales (&sc)[2], bool* fixed) {
     auto real = [](unsigned long long b) {
         double v;
         memcpy(&v, &b, sizeof(v));
         return v;
     };
-    g->fx = 1;
+    bool fx = true;
     for (int f = 0; f < 2; ++f) {
         const int recon = f ? g->recon_N : g->recon_U;
         const double err = real(scan[f].err);
@@ -239,13 +248,17 @@ hisq_status plan_links(hisq_gauge g, const LinkScan (&scan)[2], double recon_tol
         }
         for (int mu = 0; mu < 4; ++mu) {
             const double hi = real(scan[f].hi[mu]), lo = real(~scan[f].nlo[mu]);
-            int ex = 0;
-            if (hi > 0.0 && std::isfinite(hi)) std::frexp(hi, &ex);
+            int ex = kFxEmpty;
+            if (hi > 0.0 && std::isfinite(hi)) {
+                std::frexp(hi, &ex);
+                fx = fx && lo >= std::ldexp(0.2, ex) && ex >= -200 && ex <= 200 && 3 * scan[f].thin[mu] <= 18 * scan[f].links[mu];
+            }
+            fx = fx && std::isfinite(hi);
             g->fx_exp[4 * f + mu] = ex;
             sc[f].fx_exp[mu] = ex;
-            if (!std::isfinite(hi) || (hi > 0.0 && !(lo >= hi / 16.0)) || ex < -200 || ex > 200) g->fx = 0;
         }
     }
+    *fixed = fx;
     return HISQ_OK;
 }
 
@@ -266,25 +279,40 @@ hisq_status pack_links(hisq_gauge g, const double2* cu, const double2* cn, doubl
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(scan_d);
     HISQ_CUDA(e);
-    hisq_status st = plan_links(g, scan, recon_tol, sc);
+    bool fixed = false;
+    hisq_status st = plan_links(g, scan, recon_tol, sc, &fixed);
     if (st != HISQ_OK) return st;
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    size_t off[5] = {0, 0, 0, 0, 0};   // U64, N64, U_lo, N_lo
-    for (int i = 0; i < 4; ++i) {
-        const size_t nc = i < 2 ? 9 : recon[i - 2] / 2;
-        size_t sz = 2 * 4 * nc * (size_t)g->g.vh * prec_complex_bytes(i < 2 ? HISQ_F64 : g->prec);
-        if (i >= 2 && g->prec == HISQ_F64) sz = 0;
-        g->link_bytes += sz;
-        off[i + 1] = off[i] + up(sz);
+    // U64, N64, U_lo, N_lo, U_fx, N_fx
+    size_t size[6], off[7] = {0};
+    for (int i = 0; i < 6; ++i) {
+        const bool lo = i == 2 || i == 3;
+        const size_t nc = lo ? recon[i - 2] / 2 : 9;
+        size[i] = 2 * 4 * nc * (size_t)g->g.vh * prec_complex_bytes(lo ? g->prec : HISQ_F64);
+        if (lo && g->prec == HISQ_F64) size[i] = 0;
+        off[i + 1] = off[i] + ((size[i] + 255) & ~(size_t)255);
     }
-    HISQ_CUDA(cudaMalloc(&g->link_block, off[4]));
+    // the fixed-point copy is for speed only: no load fails for it, and the
+    // fields whose copies fill a good part of the device go without
+    if (size[4] + size[5] > kFxCopyMax) fixed = false;
+    e = cudaMalloc(&g->link_block, off[fixed ? 6 : 4]);
+    if (e != cudaSuccess && fixed) {
+        cudaGetLastError();
+        fixed = false;
+        e = cudaMalloc(&g->link_block, off[4]);
+    }
+    HISQ_CUDA(e);
+    for (int i = 0; i < (fixed ? 6 : 4); ++i) g->link_bytes += size[i];
     char* base = (char*)g->link_block;
     g->U64 = (double2*)base;
     g->N64 = (double2*)(base + off[1]);
     g->U_lo = g->prec == HISQ_F64 ? (void*)g->U64 : base + off[2];
     g->N_lo = g->prec == HISQ_F64 ? (void*)g->N64 : base + off[3];
-    HISQ_CUDA(launch_pack_links(g->g, cu, g->prec, g->recon_U, g->fx, sc[0], g->U64, g->U_lo, s));
-    HISQ_CUDA(launch_pack_links(g->g, cn, g->prec, g->recon_N, g->fx, sc[1], g->N64, g->N_lo, s));
+    if (fixed) {
+        g->U_fx = (int4*)(base + off[4]);
+        g->N_fx = (int4*)(base + off[5]);
+    }
+    HISQ_CUDA(launch_pack_links(g->g, cu, g->prec, g->recon_U, sc[0], g->U64, g->U_fx, g->U_lo, s));
+    HISQ_CUDA(launch_pack_links(g->g, cn, g->prec, g->recon_N, sc[1], g->N64, g->N_fx, g->N_lo, s));
     HISQ_CUDA(cudaStreamSynchronize(s));
     return HISQ_OK;
 }
@@ -569,7 +597,7 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
     }
     int r = requested ? requested : g->tune_rpt;
     if (r == 0 || r > dslash_max_rpt(prec) || n % r != 0 || n / r > 8)
-        r = prec == HISQ_F64 && g->fx ? auto_rpt_fx64(n) : auto_rpt(n, prec);
+        r = prec == HISQ_F64 && g->U_fx ? auto_rpt_fx64(n) : auto_rpt(n, prec);
     DslashTune t = dslash_default_tune(prec, r, layout);
     const int kind = kind_of_flags(g->tune_flags);
     if (!requested && g->tune_minb && r == g->tune_rpt && dslash_mapping_built(prec, r, g->tune_minb, kind) &&
@@ -625,7 +653,8 @@ void fill_common(DslashArgs& a, hisq_gauge g, int prec, int parity, int n) {
         a.lscale_u[c] = g->lscale_u[c];
         a.lscale_n[c] = g->lscale_n[c];
     }
-    a.fx = prec == HISQ_F64 ? g->fx : 0;
+    a.U_fx = prec == HISQ_F64 ? g->U_fx : nullptr;
+    a.N_fx = prec == HISQ_F64 ? g->N_fx : nullptr;
     for (int c = 0; c < 8; ++c) a.fx_exp[c] = g->fx_exp[c];
     a.red_mode = RED_NONE;
     a.finish = FIN_STORE;
@@ -1035,12 +1064,6 @@ extern "C" hisq_status hisq_apply_m(hisq_gauge g, double mass, double mu, int op
     for (int par = 0; par < 2; ++par) {
         DslashArgs a;
         fill_common(a, g, spinor_prec, par, n);
-        a.both = dslash_both_ok(a, spinor_prec);
-        for (int k = 0; k < n; ++k) {
-            a.in[k] = (const char*)v[k] + (a.both ? 0 : (1 - par) * half);
-            a.out[k] = (char*)w[k] + (a.both ? 0 : par * half);
-            a.x[k] = (const char*)v[k] + (a.both ? 0 : par * half);
-        }
         int epi = EPI_X;
         if (op == HISQ_OP_M) {
             set_mu(a, mu);
@@ -1063,6 +1086,12 @@ extern "C" hisq_status hisq_apply_m(hisq_gauge g, double mass, double mu, int op
             a.has_mu = 1;
             a.t_only = 1;
             epi = EPI_NONE;
+        }
+        a.both = dslash_both_ok(a, spinor_prec);
+        for (int k = 0; k < n; ++k) {
+            a.in[k] = (const char*)v[k] + (a.both ? 0 : (1 - par) * half);
+            a.out[k] = (char*)w[k] + (a.both ? 0 : par * half);
+            a.x[k] = (const char*)v[k] + (a.both ? 0 : par * half);
         }
         HISQ_CUDA(launch_dslash(a, spinor_prec, ru, rn, epi, t, s));
         if (a.both) break;

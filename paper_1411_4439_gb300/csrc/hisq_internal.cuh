@@ -19,6 +19,8 @@ constexpr int kMaxRhs = 16;
 constexpr int kMaxRedVals = 2 * kMaxRhs;   // per-rhs norm and max
 constexpr int kMaxRedBlocks = 4096;         // partial-sum slots per reduction finished by its last block
 constexpr int kDeferSlots = 16384;          // ... and per Dslash reduction finished by a kernel of its own
+constexpr int kFxEmpty = -300;              // exponent of a fixed-point link block without links
+constexpr size_t kFxCopyMax = 16ull << 30;  // bytes of the fixed-point copy of both link fields (64^3 x 56 sites)
 
 // ---------------------------------------------------------------------------
 // Geometry of the checkerboarded lattice
@@ -227,10 +229,10 @@ struct DslashArgs {
     int t_only;                         // 1: temporal hops only (d D / d mu)
     int l2_prefetch;                    // 1: bulk-prefetch each tile's links into L2
     int* status;                        // bounded waits that give up OR kFlagTimeout here (or null)
-    int fx;                             // 1: FP64 links in fixed point (dslash_fx64.cuh)
+    const void* U_fx;                   // FP64 links in fixed point (dslash_fx64.cuh), or null
+    const void* N_fx;
     int fx_exp[8];                      // their block exponents, [U, N][direction]
     int fx_f1[4], fx_f0[4], fx_fe[4];   // temporal factors (ft1, bt1, ft3, bt3) in limbs, set by the launcher
-    int fx_slow;                        // 1: a factor is out of range, FP64 arithmetic (set by the launcher)
     double r12_inv_scale;               // 1 / s for R12 fat links
     float lscale_u[9];                  // per-component scales of 16-bit fat links
     float lscale_n[9];                  // per-component scales of 16-bit Naik links
@@ -284,8 +286,13 @@ DslashTune dslash_default_tune(int prec, int rpt, int layout);
 DslashTune dslash_register_tune(int prec, int rpt, int layout);
 // Whether the staged-link kernel can run this lattice with `groups` groups of rpt rhs.
 bool dslash_staged_ok(const Geom& g, int prec, int rpt, int groups);
-// Whether a launch takes both parities at once (DslashArgs::both).
-inline bool dslash_both_ok(const DslashArgs& a, int prec) { return prec == HISQ_F64 && a.fx && a.red_mode == RED_NONE; }
+// Whether an FP64 launch takes the fixed-point kernel: the field has that copy
+// and the temporal factors are in its range.
+bool fx64_usable(const DslashArgs& a);
+// Whether a launch takes both parities at once (DslashArgs::both); ask once the factors are set.
+inline bool dslash_both_ok(const DslashArgs& a, int prec) {
+    return prec == HISQ_F64 && a.red_mode == RED_NONE && fx64_usable(a);
+}
 // Largest rhs-per-thread value instantiated for a precision.
 int dslash_max_rpt(int prec);
 // Bundle layout: rhs per 16-byte chunk of a storage precision (F32: 2,
@@ -304,27 +311,28 @@ cudaError_t launch_transpose_spinor(const double2* in, double2* out, int n, int 
 // ---------------------------------------------------------------------------
 // Link packing (gauge.cu)
 // ---------------------------------------------------------------------------
-// What one pass over a canonical field finds (all values are the bits of
+// What one pass over a canonical field finds (comp to err are the bits of
 // non-negative doubles): the largest |Re|, |Im| of every stored component
 // (recon / 2 of them), per direction the largest over all reals and the
 // complement of the smallest over nonzero links of a link's largest (0 if
-// there is none), and the largest reconstruct error.
+// there is none), and the largest reconstruct error; per direction the number
+// of nonzero links and of their reals below 1/16 of the link's largest.
 struct LinkScan {
-    unsigned long long comp[9], hi[4], nlo[4], err;
+    unsigned long long comp[9], hi[4], nlo[4], err, links[4], thin[4];
 };
 cudaError_t launch_link_scan(const Geom& g, const double2* canon, int recon, int hop, double r12_inv_scale,
                              LinkScan* out, cudaStream_t s);
-// Pack canonical complex128 [4][V][3][3] into the FP64 copy out64 [2][4][9][vh]
-// (doubles, or with fx int4 limbs (re1, re0, im1, im0) of value 2^(55 - sc.fx_exp[mu]),
-// see dslash_fx64.cuh) and, for F32 / F16, into the storage copy out_lo
-// [2][4][recon / 2][vh]. F16 links are 16-bit fixed point, value * sc.inv[c]
-// rounded for stored component c.
+// Pack canonical complex128 [4][V][3][3] into the FP64 copy out64 [2][4][9][vh],
+// unless null into its fixed-point form out_fx (int4 limbs (re1, re0, im1, im0)
+// of value 2^(55 - sc.fx_exp[mu]), see dslash_fx64.cuh) and, for F32 / F16, into
+// the storage copy out_lo [2][4][recon / 2][vh]. F16 links are 16-bit fixed
+// point, value * sc.inv[c] rounded for stored component c.
 struct LinkScales {
     int fx_exp[4];
     double inv[9];
 };
-cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, int fx, const LinkScales& sc,
-                              void* out64, void* out_lo, cudaStream_t s);
+cudaError_t launch_pack_links(const Geom& g, const double2* canon, int prec, int recon, const LinkScales& sc, void* out64,
+                              void* out_fx, void* out_lo, cudaStream_t s);
 // Compress to double [4][V][r] and back (ABI helpers).
 cudaError_t launch_compress_links(const Geom& g, const double2* canon, int recon, int hop,
                                   double r12_inv_scale, double* packed,
