@@ -116,10 +116,10 @@ const char* hisq_last_error(void);
  * bytes again; a load that cannot get them does without) and FP64 operators
  * sum in fixed point relative to the largest neighbour of a site, scaled by the
  * field's largest link. An output real that is small against that is summed in
- * FP64 from the FP64 copy. Sites are no further off than with FP64 multiply-adds;
- * a real alone is within 1600 x 2^-53 of the sum of its |products| (typically
- * 0.2 x 2^-53), where 96 multiply-adds stay within 96 x 2^-53. Links or vectors that are not finite take
- * FP64 multiply-adds.
+ * FP64 from the FP64 copy. A real is within 1600 x 2^-53 of the sum of its
+ * |products| (typically 0.2 x 2^-53), where 96 FP64 multiply-adds stay within
+ * 96 x 2^-53 (typically 0.6 x 2^-53). Links or vectors that are not finite, and
+ * |mu| beyond about 13, take FP64 multiply-adds.
  * prec == HISQ_F16 stores every link real as a 16-bit integer q with value
  * q * s_c, one scale s_c = max |Re|,|Im| / 32767 per stored complex
  * component c of each field (2^-15 of the range, where IEEE half keeps only

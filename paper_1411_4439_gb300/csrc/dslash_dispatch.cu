@@ -184,6 +184,10 @@ static int fx64_split(const DslashArgs& a, int rpt) {
     return rpt <= 2 && warps < 4ll * device_sm_count() ? 4 : 1;
 }
 
+// A hop's scale 2^o (link block and temporal factor) below 2^64 keeps zeros
+// and subnormal reals out of the fixed-point sums (fx_limbs gives every real a
+// leading bit and needs 64 bits of shift to drop it); loading a field bounds
+// its blocks by 2^60, so only |mu| beyond about 13 leaves the range.
 bool fx64_usable(const DslashArgs& a) {
     if (a.U_fx == nullptr || a.N_fx == nullptr) return false;
     if (!a.has_mu) return true;
@@ -192,7 +196,7 @@ bool fx64_usable(const DslashArgs& a) {
         if (!std::isfinite(f[i]) || f[i] == 0.0) return false;
         int e = 0;
         std::frexp(f[i], &e);
-        if (e <= -400 || e >= 400) return false;
+        if (e < -400 || a.fx_exp[(i >> 1) * 4 + 3] + e > 64) return false;
     }
     return true;
 }

@@ -419,14 +419,15 @@ struct FxHops {
         }
     }
 
-    // Whether rhs j needs FP64 arithmetic: a neighbour too large, or an output real whose sums stayed below 2^(E - kFxReach). (Neighbours
+    // Whether rhs j needs FP64 arithmetic: a neighbour that is not finite or too
+    // large, or an output real whose sums stayed below 2^(E - kFxReach). (Neighbours
     // that are all zero give exact zeros.)
     __device__ __forceinline__ bool rare(int j) const {
         constexpr unsigned kSmall = (1u << (23 - kFxReach - 16)) - 1;   // hi word of 2^(E - kFxReach) is 2^(23 - kFxReach)
         bool low = false;
 #pragma unroll
         for (int i = 0; i < 3; ++i) low = low || (tops[j][i] & 0xffffu) <= kSmall || (tops[j][i] >> 16) <= kSmall;
-        return E[j] > kFxCeil || (low && peak[j] != 0u);
+        return peak[j] >= 0xffe00000u || E[j] > kFxCeil || (low && peak[j] != 0u);
     }
 
     // (S2 2^28 + S1) 2^(E - 83), times sgn = +-1

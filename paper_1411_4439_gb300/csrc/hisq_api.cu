@@ -251,7 +251,7 @@ hisq_status plan_links(hisq_gauge g, const LinkScan (&scan)[2], double recon_tol
             int ex = kFxEmpty;
             if (hi > 0.0 && std::isfinite(hi)) {
                 std::frexp(hi, &ex);
-                fx = fx && lo >= std::ldexp(0.2, ex) && ex >= -200 && ex <= 200 && 3 * scan[f].thin[mu] <= 18 * scan[f].links[mu];
+                fx = fx && lo >= std::ldexp(0.2, ex) && ex >= -200 && ex <= 60 && 3 * scan[f].thin[mu] <= 18 * scan[f].links[mu];
             }
             fx = fx && std::isfinite(hi);
             g->fx_exp[4 * f + mu] = ex;

@@ -191,3 +191,40 @@ def test_full_lattice_operators_keep_the_bits_of_every_real(gpu_lib, kind):
                 within(got[:, p * half:(p + 1) * half], ref, size, 102)
     finally:
         H.hisq_gauge_free(g)
+
+
+@pytest.mark.parametrize("mu", [-60.0, -30.0, -16.0, -5.0, 5.0, 12.0, 16.0, 20.0, 30.0, 60.0])
+def test_large_temporal_factors(gpu_lib, mu):
+    """Zero stays zero, non-finite neighbours are seen behind any factor, the rest keeps its bits."""
+    L, n = (4, 6, 8, 10), 2
+    U, N, v = structured("haar", L, n, seed=33)
+    v = np.ascontiguousarray(v[:, v.shape[1] // 2:])
+    g = load(gpu_lib, L, U, N)
+    try:
+        ref, size = exact(U, N, v, L, 0, exp_factors(mu))
+        within(dslash(gpu_lib, g, v, 0, mu), ref, size, 102)
+        assert not dslash(gpu_lib, g, 0.0 * v, 0, mu).any()
+        for bad in (np.inf, -np.inf, np.nan):
+            w = v.copy()
+            w[n - 1, 17, 1] = bad
+            with np.errstate(invalid="ignore"):
+                want = np.isfinite(O.dslash_parity(U, N, w, L, 0, mu))
+            got = dslash(gpu_lib, g, w, 0, mu)
+            assert (np.isfinite(got) == want).all() and not want.all()
+    finally:
+        gpu_lib.hisq_gauge_free(g)
+
+
+def test_small_and_large_links(gpu_lib):
+    """Fields of size 2^-150 to 2^150, and zero vectors on them."""
+    L, n = (4, 6, 8, 10), 2
+    for scale in (-150, -70, 40, 62, 90, 120, 150):
+        U, N, v = structured("haar", L, n, seed=34)
+        U, N, v = 2.0 ** scale * U, 2.0 ** scale * N, np.ascontiguousarray(v[:, v.shape[1] // 2:])
+        g = load(gpu_lib, L, U, N)
+        try:
+            ref, size = exact(U, N, v, L, 0, exp_factors(0.0))
+            within(dslash(gpu_lib, g, v, 0), ref, size, 96)
+            assert not dslash(gpu_lib, g, 0.0 * v, 0).any()
+        finally:
+            gpu_lib.hisq_gauge_free(g)
