@@ -113,6 +113,8 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* bits, doub
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
+constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;
+__device__ __forceinline__ unsigned long long skip_nan(unsigned long long b) { return b > kInfBits ? 0ull : b; }
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
     return a > b ? a : b;
 }
@@ -174,9 +176,18 @@ __global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __rest
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
             m[c] = src[c];
-            const unsigned long long b = umax64(abs_bits(m[c].x), abs_bits(m[c].y));
-            if (c < NC && (c < 6 || RECON == 18)) mx[c] = umax64(mx[c], b);
-            link = umax64(link, b);
+            link = umax64(link, umax64(abs_bits(m[c].x), abs_bits(m[c].y)));
+        }
+        // a NaN is its own link's matter: the scales of the others come from the numbers
+        const bool nan = link > kInfBits;
+#pragma unroll
+        for (int c = 0; c < NC && (c < 6 || RECON == 18); ++c) {
+            unsigned long long x = abs_bits(m[c].x), y = abs_bits(m[c].y);
+            if (nan) {
+                x = skip_nan(x);
+                y = skip_nan(y);
+            }
+            mx[c] = umax64(mx[c], umax64(x, y));
         }
         hi = umax64(hi, link);
         if (link != 0ull) {
@@ -191,7 +202,7 @@ __global__ void __launch_bounds__(256) scan_kernel(Geom g, const double2* __rest
         if (RECON != 18) {
             const int sg = RECON == 12 ? staggered_sign(g, site_of(g, i), mu, hop) : 1;
             const double2 f = third_factor<RECON>(m, sg, inv_s, err);
-            if (RECON == 14) mx[NC - 1] = umax64(mx[NC - 1], umax64(abs_bits(f.x), abs_bits(f.y)));
+            if (RECON == 14) mx[NC - 1] = umax64(mx[NC - 1], umax64(skip_nan(abs_bits(f.x)), skip_nan(abs_bits(f.y))));
         }
     }
     __shared__ unsigned long long s_v[12][8];
@@ -266,9 +277,9 @@ __device__ __forceinline__ int2 fx_split(double v, int e) {
     return make_int2((int)((q - lo) >> 28), lo);
 }
 
-// 16-bit fixed point: round to nearest of v / scale, clamped to +-32767
+// 16-bit fixed point: round to nearest of v / scale, clamped to +-32767 (NaN: -32767)
 __device__ __forceinline__ short quantize(double v, double inv_scale) {
-    const int q = __double2int_rn(v * inv_scale);
+    const int q = abs_bits(v) > kInfBits ? -32767 : __double2int_rn(v * inv_scale);
     return (short)min(max(q, -32767), 32767);
 }
 __device__ __forceinline__ float4 store_pair(double2 a, double2 b, const double*, int, float2) {
