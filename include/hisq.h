@@ -161,6 +161,8 @@ hisq_status hisq_gauge_info(hisq_gauge g, int L[4], hisq_prec* prec,
  * two hops in flight while the current hop is multiplied (FP32/FP16). At
  * most one of PACKED, STAGED, PIPELINED, PIPELINED2. Mappings that are not
  * built or do not fit n or the lattice fall back to the automatic choice.
+ * FP64 calls on a field kept in fixed point (see hisq_gauge_load) take the rhs
+ * per thread alone.
  */
 enum {
     HISQ_MAP_PACKED = 1,

@@ -201,6 +201,9 @@ bool fx64_usable(const DslashArgs& a) {
     return true;
 }
 
+// The instances of dslash_fx64_inst.cu.
+int fx64_min_blocks(int rpt, int n) { return rpt == 1 ? 2 : rpt == 2 && n <= 4 * rpt ? 3 : 1; }
+
 cudaError_t launch_dslash(const DslashArgs& a, int prec, int ru, int rn, int epi,
                           const DslashTune& t, cudaStream_t s) {
     if (!dslash_variant_supported(prec, ru, rn, epi)) return cudaErrorInvalidValue;

@@ -193,7 +193,7 @@ struct hisq_gauge_s {
     int tune_rpt = 0;            // 0 = automatic
     int tune_minb = 0;
     int tune_flags = 0;          // HISQ_MAP_* bits
-    std::map<int, DslashTune> tuned;   // autotuned mappings by tuned_key(n, prec, layout)
+    std::map<int, DslashTune> tuned;   // autotuned mappings by tuned_key(g, n, prec, layout)
     void* mdagm_tmp = nullptr;
     size_t mdagm_tmp_bytes = 0;
     double* dot_partials = nullptr;     // reduction scratch of hisq_cdot
@@ -523,7 +523,11 @@ int auto_rpt(int n, int prec) {
     return r;
 }
 
-int tuned_key(int n, int prec, int layout) { return n * 100 + prec * 10 + layout; }
+// FP64 calls run another kernel on a field with fixed-point links, and the
+// tuned mappings of a shape are kept for later fields of either kind.
+int tuned_key(hisq_gauge g, int n, int prec, int layout) {
+    return n * 100 + prec * 10 + layout + (prec == HISQ_F64 && g->U_fx ? 10000 : 0);
+}
 
 int kind_of_flags(int flags) {
     if (flags & HISQ_MAP_PACKED) return KIND_PACKED;
@@ -567,7 +571,7 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
     if (layout == HISQ_BUNDLE) {
         // the bundle kernel (rpt 0 when n does not fit the layout)
         if (!requested && g->tune_rpt == 0 && g->tune_flags == 0) {
-            auto it = g->tuned.find(tuned_key(n, prec, layout));
+            auto it = g->tuned.find(tuned_key(g, n, prec, layout));
             if (it != g->tuned.end()) return it->second;
         }
         DslashTune t = dslash_bundle_tune(prec, n);
@@ -592,7 +596,7 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
         return t;
     }
     if (!requested && g->tune_rpt == 0 && g->tune_flags == 0) {
-        auto it = g->tuned.find(tuned_key(n, prec, layout));
+        auto it = g->tuned.find(tuned_key(g, n, prec, layout));
         if (it != g->tuned.end()) return it->second;
     }
     int r = requested ? requested : g->tune_rpt;
@@ -605,7 +609,7 @@ DslashTune pick_tune(hisq_gauge g, int n, int prec, int requested, int layout) {
         t.minb = g->tune_minb;
         t.kind = kind;
     }
-    if (g->tune_flags & HISQ_MAP_L2_PREFETCH) t.prefetch = 1;
+    if ((g->tune_flags & HISQ_MAP_L2_PREFETCH) && !(prec == HISQ_F64 && g->U_fx)) t.prefetch = 1;
     return t;
 }
 
@@ -621,7 +625,7 @@ extern "C" hisq_status hisq_get_dslash_mapping_ex(hisq_gauge g, int n, hisq_prec
     const DslashTune t = pick_tune(g, n, prec, 0, layout);
     if (layout == HISQ_BUNDLE && t.rpt == 0) return fail(HISQ_EINVAL, "no bundle kernel for n = %d", n);
     if (rpt) *rpt = t.rpt;
-    if (minb) *minb = t.minb;
+    if (minb) *minb = prec == HISQ_F64 && g->U_fx ? fx64_min_blocks(t.rpt, n) : t.minb;
     if (flags) *flags = flags_of_tune(t);
     return HISQ_OK;
 }
@@ -922,7 +926,7 @@ extern "C" hisq_status hisq_autotune_dslash(hisq_gauge g, int n, hisq_prec prec,
         }
     }
     cleanup();
-    g->tuned[tuned_key(n, prec, layout)] = best_t;
+    g->tuned[tuned_key(g, n, prec, layout)] = best_t;
     if (rpt) *rpt = best_t.rpt;
     if (minb) *minb = best_t.minb;
     if (flags) *flags = flags_of_tune(best_t);

@@ -289,6 +289,8 @@ bool dslash_staged_ok(const Geom& g, int prec, int rpt, int groups);
 // Whether an FP64 launch takes the fixed-point kernel: the field has that copy
 // and the temporal factors are in its range.
 bool fx64_usable(const DslashArgs& a);
+// Blocks per SM that kernel is compiled for with n rhs, rpt per thread.
+int fx64_min_blocks(int rpt, int n);
 // Whether a launch takes both parities at once (DslashArgs::both); ask once the factors are set.
 inline bool dslash_both_ok(const DslashArgs& a, int prec) {
     return prec == HISQ_F64 && a.red_mode == RED_NONE && fx64_usable(a);
