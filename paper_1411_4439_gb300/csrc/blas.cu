@@ -106,7 +106,7 @@ __device__ bool block_reduce_arrive(const RedScratch& red, R (&val)[NV], int n, 
         red.partials[(size_t)(blockIdx.y * NV + j) * kMaxRedBlocks + blockIdx.x] = acc;
     }
     if (!last_block_arrive(red.counter, gridDim.x * gridDim.y)) return false;
-    finish_values(red, n * NV, gridDim.x, [](int v) { return (NV == 2) && (v & 1); }, s_vals);
+    finish_values<8>(red, n * NV, gridDim.x, [](int v) { return (NV == 2) && (v & 1); }, s_vals);
     return true;
 }
 

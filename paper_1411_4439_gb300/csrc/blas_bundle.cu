@@ -109,7 +109,7 @@ __device__ bool group_reduce_arrive(const RedScratch& red, float (&val)[NV], int
         red.partials[(size_t)(blockIdx.y * NV + j) * kMaxRedBlocks + blockIdx.x] = acc;
     }
     if (!last_block_arrive(red.counter, gridDim.x * gridDim.y)) return false;
-    finish_values(red, groups * NV, gridDim.x, [](int) { return false; }, s_vals);
+    finish_values<8>(red, groups * NV, gridDim.x, [](int) { return false; }, s_vals);
     return true;
 }
 

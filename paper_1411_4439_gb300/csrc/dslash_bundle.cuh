@@ -37,6 +37,8 @@
 // (visit_site), so the neighbour chunks stay in L2 between their readers.
 #pragma once
 
+#include <type_traits>
+
 #include "dslash_impl.cuh"
 
 namespace hisq {
@@ -1045,7 +1047,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_bundle_kernel(const DslashAr
         if (EPI == EPI_X && a.red_mode != RED_NONE) tile_reduce<R>(a, k0, red0, red0, parts, it == 0);
     }
     if (a.red_mode == RED_NONE) return;
-    block_finish(a, parts);
+    block_finish<std::is_same<S, float>::value>(a, parts);
 }
 
 // Whether (n, rhs per thread) fits the bundle kernel of storage S.
@@ -1091,7 +1093,7 @@ cudaError_t launch_dslash_bundle(const DslashArgs& args, cudaStream_t s) {
         e = cached_occupancy(cache, kern, bx * G, smem, G, &occ);
         if (e != cudaSuccess) return e;
     }
-    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + bx - 1) / bx);
+    const unsigned blocks = plan_tiles<std::is_same<S, float>::value>(a, ((long long)a.g.vh + bx - 1) / bx);
     kern<<<blocks, block, smem, s>>>(a);
     return finish_launch(a, blocks, s);
 }

@@ -515,7 +515,9 @@ __global__ void __launch_bounds__(MAXT, MINB) dslash_fx64_kernel(const __grid_co
 #pragma unroll
         for (int j = 0; j < R; ++j) red1[j] = sqrt(red1[j]);
     }
-    block_reduce_finish<R>(a, k0, red0, red1);
+    __shared__ RedParts parts;
+    tile_reduce<R>(a, k0, red0, red1, parts, true);
+    block_finish<false>(a, parts);
 }
 
 // Temporal factor f (in fx64_usable's range) as a 55-bit mantissa in limbs and an exponent.
@@ -551,7 +553,7 @@ cudaError_t launch_fx64(const DslashArgs& args, cudaStream_t s) {
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
     const int spb = bx / SPLIT;
-    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + spb - 1) / spb);
+    const unsigned blocks = plan_tiles<false>(a, ((long long)a.g.vh + spb - 1) / spb);
     kern<<<dim3(blocks, a.both ? 2 : 1), dim3(bx, G), 0, s>>>(a);
     return finish_launch(a, blocks, s);
 }

@@ -10,6 +10,8 @@
 // per-rhs reductions the CG needs (Re<x,out> or |out|^2 and max|out_i|).
 #pragma once
 
+#include <type_traits>
+
 #include <atomic>
 
 #include "hisq_internal.cuh"
@@ -292,7 +294,7 @@ __device__ __forceinline__ int wrap(int c, int L) {
 template <typename SC, int RPT, int EPI, int LAYOUT, typename R, typename RC>
 __device__ __forceinline__ void epilogue_site(const DslashArgs& a, int h, int k0, const RC (&acc)[RPT][3],
                                               R (&red0)[RPT], R (&red1)[RPT]);
-template <int RPT, typename R>
+template <int RPT, bool MULTI = false, typename R>
 __device__ __forceinline__ void block_reduce_finish(const DslashArgs& a, int k0, R (&red0)[RPT],
                                                     R (&red1)[RPT]);
 
@@ -428,7 +430,7 @@ __global__ void __launch_bounds__(256, MINB) dslash_kernel(const DslashArgs a) {
     }
 
     if (a.red_mode == RED_NONE) return;
-    block_reduce_finish<RPT>(a, k0, red0, red1);
+    block_reduce_finish<RPT, LAYOUT == HISQ_SOA && std::is_same<S, float>::value>(a, k0, red0, red1);
 }
 
 // Epilogue of one output site: out = [y] + cx x + cd (D in) for the thread's
@@ -509,11 +511,11 @@ __device__ __forceinline__ void tile_reduce(const DslashArgs& a, int k0, R (&red
     }
 }
 
-// The block's sums into its partial slot. With a.red_defer the sums over the
-// blocks and the finish are left to launch_red_finish; else the last block
-// does them. Called by every thread of the block.
+// The block's sums into its partial slots. The sums over the blocks and the
+// finish are launch_red_finish's, or with LAST and few blocks (a.red_defer 0)
+// the last block's. Called by every thread of the block.
+template <bool LAST>
 __device__ __forceinline__ void block_finish(const DslashArgs& a, const RedParts& parts) {
-    __shared__ double s_vals[kMaxRedVals];
     const int nv = (a.red_mode == RED_NORM_MAX_W) ? 2 : 1;
     const int wpg = (blockDim.x + 31) >> 5;      // warps per group
     __syncthreads();
@@ -523,22 +525,51 @@ __device__ __forceinline__ void block_finish(const DslashArgs& a, const RedParts
         const bool is_max = (nv == 2) && (tid & 1);
         double acc = 0.0;
         for (int w = 0; w < wpg; ++w) acc = is_max ? fmax(acc, parts.v[tid][w]) : acc + parts.v[tid][w];
-        a.red.partials[(size_t)tid * (a.red_defer ? kDeferSlots : kMaxRedBlocks) + blockIdx.x] = acc;
+        a.red.partials[(size_t)tid * (!LAST || a.red_defer ? kDeferSlots : kMaxRedBlocks) + blockIdx.x] = acc;
     }
-    if (a.red_defer) return;
-    if (!last_block_arrive(a.red.counter, gridDim.x)) return;
-    finish_values(a.red, nvals, gridDim.x, [nv](int v) { return nv == 2 && (v & 1); }, s_vals);
-    if (tid < a.nrhs)
-        finish_rhs(a.finish, a.cg, a.red_out, tid, nv, s_vals[tid * nv], nv == 2 ? s_vals[tid * nv + 1] : 0.0, a.tol2,
-                   fin_load(a.cg, tid));
+    if constexpr (LAST) {
+        __shared__ double s_vals[kMaxRedVals];
+        if (a.red_defer) return;
+        if (!last_block_arrive(a.red.counter, gridDim.x)) return;
+        finish_values(a.red, nvals, gridDim.x, [nv](int v) { return nv == 2 && (v & 1); }, s_vals);
+        if (tid >= a.nrhs) return;
+        if (a.finish == FIN_CG_ALPHA) {
+            finish_cg_alpha(a.cg, tid, s_vals[tid], fin_load(a.cg, tid));
+        } else if (a.finish == FIN_RELIABLE) {
+            finish_reliable(a.cg, tid, s_vals[2 * tid], s_vals[2 * tid + 1], a.tol2);
+        } else if (a.red_out != nullptr) {
+            for (int v = 0; v < nv; ++v) a.red_out[tid * nv + v] = s_vals[tid * nv + v];
+        }
+    }
 }
 
-template <int RPT, typename R>
+// Warp sums and the block's end in the kernels on the per-rhs layouts, whose
+// main loops fill their registers: with tile_reduce here (MULTI), finish_rhs and
+// eight slots in flight in the last block, calls without a reduction ran 2 to 15 %
+// slower (20x28x36x10, F32, n = 5: 44.2 us against 41.2; R12 / R14, n = 8: 15 %).
+// The F32 register kernels on the SoA layout alone are 1 to 4 % faster with it.
+template <int RPT, bool MULTI, typename R>
 __device__ __forceinline__ void block_reduce_finish(const DslashArgs& a, int k0, R (&red0)[RPT],
                                                     R (&red1)[RPT]) {
     __shared__ RedParts parts;
-    tile_reduce<RPT>(a, k0, red0, red1, parts, true);
-    block_finish(a, parts);
+    if constexpr (MULTI) {
+        tile_reduce<RPT>(a, k0, red0, red1, parts, true);
+        block_finish<true>(a, parts);
+        return;
+    }
+    const int nv = (a.red_mode == RED_NORM_MAX_W) ? 2 : 1;
+    const int lane = threadIdx.x & 31;
+    const int wig = threadIdx.x >> 5;            // warp index within the group
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+        const double s0 = (double)warp_sum(red0[j]);
+        const double s1 = (double)warp_max(red1[j]);
+        if (lane == 0) {
+            parts.v[(k0 + j) * nv][wig] = s0;
+            if (nv == 2) parts.v[(k0 + j) * nv + 1][wig] = s1;
+        }
+    }
+    block_finish<true>(a, parts);
 }
 
 // Resident blocks per SM of one kernel, cached per device: every launcher
@@ -605,17 +636,27 @@ cudaError_t cached_occupancy(OccCache& cache, K* kern, int threads, size_t smem,
 // order that the L2 reuse rests on (strided tiles: 64^3x16, n = 4, FP32 452 us
 // against 392).
 //
-// The sums over the blocks: with many blocks, a kernel of its own after the
-// launch (launch_red_finish). Finding the last block costs every block a fence
-// over its stores and an atomic round trip while it holds its slot (32^3x8,
-// n = 8, FP32, second Dslash of the CG: 59 us against 43 without the sums).
-// Few blocks (kInlineBlocks) run side by side, and the launch costs more.
+// The sums over the blocks: a kernel of its own after the launch
+// (launch_red_finish). Finding the last block costs every block a fence over
+// its stores and an atomic round trip while it holds its slot (32^3x8, n = 8,
+// FP32, second Dslash of the CG: 59 us against 43 without the sums), and with
+// few blocks the round trip and the sum are no shorter than a launch. CG
+// iteration with the last block up to 1024 blocks, up to 128 and never: 8^4,
+// FP32, n = 8: 28.7, 28.7 and 28.0 us; 16^3x8, FP16, n = 8: 43.6, 43.6 and 42.2;
+// 8^4, FP64, n = 1: 26.1, 26.3 and 25.4; 20x28x36x10, FP32, n = 8: 118, 109, 109.
+//
+// The per-rhs and FP32 bundle kernels (LAST) keep the last block up to
+// kInlineBlocks all the same, for the compiler's sake: without that code behind
+// it their main loop is allotted and scheduled worse (FP32, 48^3x12, n = 8,
+// second Dslash of the CG: 223.5 us and 230.7; 20x28x36x10, n = 8: 44.9 and 45.7;
+// FP16 the other way round: 198.5 and 195.0).
 constexpr int kInlineBlocks = 128;
+template <bool LAST>
 inline unsigned plan_tiles(DslashArgs& a, long long tiles) {
     a.run = 1;
     if (a.red_mode != RED_NONE) a.run = (int)((tiles + kDeferSlots - 1) / kDeferSlots);
     const long long blocks = (tiles + a.run - 1) / a.run;
-    a.red_defer = a.red_mode != RED_NONE && blocks > kInlineBlocks;
+    a.red_defer = a.red_mode != RED_NONE && !(LAST && blocks <= kInlineBlocks);
     return (unsigned)blocks;
 }
 inline cudaError_t finish_launch(const DslashArgs& a, unsigned blocks, cudaStream_t s) {
@@ -639,12 +680,15 @@ cudaError_t launch_dslash_instance(const DslashArgs& args, cudaStream_t s) {
     int occ = 0;
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
-    // one resident wave (a block per tile: 20x28x36x10, n = 6, FP32 1 % slower)
+    // One resident wave with strided tiles. A block per tile against it, 20x28x36x10 /
+    // 32^3x8 / 48^3x12: FP32 n = 6, 7 and 14 1 to 3 % slower, n = 3 and 5 11 to 27 %
+    // faster; FP16 n = 2 0 / 5 % slower / 5 % faster, n = 3, 5, 7 and 14 8 to 20 % faster;
+    // no rule on sizes has been found that takes the gains without the losses.
     long long tiles = ((long long)a.g.vh + bx - 1) / bx;
     const long long cap = (long long)occ * device_sm_count();
     if (tiles > cap) tiles = cap;
     if (tiles > kMaxRedBlocks) tiles = kMaxRedBlocks;
-    const unsigned blocks = plan_tiles(a, tiles);
+    const unsigned blocks = plan_tiles<true>(a, tiles);
     kern<<<blocks, block, 0, s>>>(a);
     return finish_launch(a, blocks, s);
 }

@@ -11,6 +11,8 @@
 // Temporal-only operators (d^n D / d mu^n) are not routed here.
 #pragma once
 
+#include <type_traits>
+
 #include "dslash_impl.cuh"
 
 namespace hisq {
@@ -199,6 +201,15 @@ __device__ __forceinline__ void epilogue_site_px(const DslashArgs& a, int h, int
     }
 }
 
+// Blocks take consecutive tiles (RUN), or strided ones, of which a block has
+// one where the grid covers the lattice. How the compiler allots the registers
+// of the pipeline differs by the form of the loop, on all lattices alike (8^4 to
+// 48^3x12): consecutive tiles are 4 to 9 % faster in the two instances here,
+// strided ones up to 15 % in all others (F32, R12 or R14 fat links).
+template <typename S, int RU, int RN, int EPI, int LAYOUT>
+constexpr bool kPipeRuns = EPI == EPI_NONE && ((std::is_same<S, float>::value && RU == 18 && RN == 18 && LAYOUT == HISQ_AOS) ||
+                                               (std::is_same<S, __half>::value && RU == 18 && RN == 14 && LAYOUT == HISQ_SOA));
+
 template <typename S, typename LS, int RU, int RN, int RPT, int MINB, int DEPTH, int EPI, int LAYOUT>
 __global__ void __launch_bounds__(256, MINB) dslash_pipe_kernel(const DslashArgs a) {
     using R = typename Traits<S>::R;
@@ -213,8 +224,10 @@ __global__ void __launch_bounds__(256, MINB) dslash_pipe_kernel(const DslashArgs
         red0[j] = (R)0;
         red1[j] = (R)0;
     }
-    const int v0 = blockIdx.x * a.run * blockDim.x;
-    for (int it = 0, v = v0 + threadIdx.x; it < a.run && v - (int)threadIdx.x < vh; ++it, v += blockDim.x) {
+    constexpr bool RUN = kPipeRuns<S, RU, RN, EPI, LAYOUT>;
+    const int v0 = RUN ? blockIdx.x * a.run * blockDim.x : blockIdx.x * blockDim.x;
+    const int step = RUN ? blockDim.x : gridDim.x * blockDim.x;
+    for (int it = 0, v = v0 + threadIdx.x; (!RUN || it < a.run) && v - (int)threadIdx.x < vh; ++it, v += step) {
         if (v >= vh) continue;
         const int h = visit_site(v, a.g);
         RC acc[RPT][3];
@@ -259,7 +272,18 @@ cudaError_t launch_dslash_pipe(const DslashArgs& args, cudaStream_t s) {
     int occ = 0;
     cudaError_t e = cached_occupancy(cache, kern, bx * G, 0, G, &occ);
     if (e != cudaSuccess) return e;
-    const unsigned blocks = plan_tiles(a, ((long long)a.g.vh + bx - 1) / bx);
+    // One resident wave with strided tiles while a block has few of them, a block
+    // per tile from eight on: 32^3x8, n = 8, FP16 (3.4 waves): 49.8 and 50.9 us;
+    // 48^3x12 (17 waves): 263 and 241, where strided tiles lose the reuse in L2.
+    // Three rhs groups with full fat links stay with the wave (48^3x12, n = 12,
+    // FP16: 395 and 403 us; R12 fat links, SoA, F32: 494 and 456), with compressed
+    // ones in FP16 they leave it at four (20x28x36x10, 5.2 waves, R14: 72.4 and 62.0).
+    const int many = std::is_same<S, __half>::value && G > 2 ? 4 : 8;
+    long long tiles = ((long long)a.g.vh + bx - 1) / bx;
+    const long long cap = (long long)occ * device_sm_count();
+    const bool wave = (G > 2 && RU == 18) || tiles < many * cap || (a.red_mode != RED_NONE && tiles > kDeferSlots);
+    if (!kPipeRuns<S, RU, RN, EPI, LAYOUT> && wave && tiles > cap) tiles = cap;
+    const unsigned blocks = plan_tiles<true>(a, tiles);
     kern<<<blocks, block, 0, s>>>(a);
     return finish_launch(a, blocks, s);
 }

@@ -351,7 +351,8 @@ inline bool staged_geometry_ok(const Geom& g, size_t elem) {
 }
 
 template <typename S, typename LS, int RU, int RN, int RPT, int MINB, int EPI, int LAYOUT>
-cudaError_t launch_dslash_staged(const DslashArgs& a, cudaStream_t s) {
+cudaError_t launch_dslash_staged(const DslashArgs& args, cudaStream_t s) {
+    DslashArgs a = args;
     using LC = typename Traits<LS>::C;
     constexpr int NCU = (RU == 18) ? 9 : (RU == 14 ? 7 : 6);
     constexpr int NCN = (RN == 18) ? 9 : (RN == 14 ? 7 : 6);
@@ -369,8 +370,9 @@ cudaError_t launch_dslash_staged(const DslashArgs& a, cudaStream_t s) {
     const long long cap = (long long)occ * device_sm_count();
     if (nblk > cap) nblk = cap;
     if (nblk > kMaxRedBlocks) nblk = kMaxRedBlocks;
-    kern<<<(unsigned)nblk, block, smem, s>>>(a);
-    return cudaGetLastError();
+    const unsigned blocks = plan_tiles<true>(a, nblk);
+    kern<<<blocks, block, smem, s>>>(a);
+    return finish_launch(a, blocks, s);
 }
 
 }  // namespace hisq

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kDotThreads) cdot_kernel(ForcePtrs vw, long lo
         red.partials[(size_t)(k * 2 + threadIdx.x) * kMaxRedBlocks + blockIdx.x] = acc;
     }
     if (!last_block_arrive(red.counter, gridDim.x * gridDim.y)) return;
-    finish_values(red, 2 * n, gridDim.x, [](int) { return false; }, s_vals);
+    finish_values<8>(red, 2 * n, gridDim.x, [](int) { return false; }, s_vals);
     if (threadIdx.x < 2 * n) out[threadIdx.x] = s_vals[threadIdx.x];
 }
 

@@ -144,10 +144,11 @@ __device__ __forceinline__ void st_c(float2* p, float2 v) { *p = v; }
 __device__ __forceinline__ void st_c(__half2* p, float2 v) { *p = __float22half2_rn(v); }
 
 // ---------------------------------------------------------------------------
-// Reductions: per-block partials and a last-block finish in fixed order
+// Reductions: per-block partials, summed in fixed order by the last block or,
+// after a Dslash of many blocks, by a kernel of its own
 // ---------------------------------------------------------------------------
 struct RedScratch {
-    double* partials;        // [kMaxRedVals][kMaxRedBlocks]
+    double* partials;        // [kMaxRedVals][kMaxRedBlocks], of a deferred reduction [kMaxRedVals][kDeferSlots]
     unsigned int* counter;   // zero between launches; the last block resets it
 };
 
@@ -214,8 +215,6 @@ enum Finish : int {
 struct DslashArgs {
     Geom g;
     int parity;                         // output parity
-    int both;                           // 1: both parities in one launch (F64 fixed-point links, no reduction):
-                                        // in, out, x, y are parity-blocked full-lattice vectors
     int nrhs;                           // rhs in this launch
     const void* U;                      // packed links, [2][4][ncomp][vh]
     const void* N;
@@ -229,10 +228,6 @@ struct DslashArgs {
     int t_only;                         // 1: temporal hops only (d D / d mu)
     int l2_prefetch;                    // 1: bulk-prefetch each tile's links into L2
     int* status;                        // bounded waits that give up OR kFlagTimeout here (or null)
-    const void* U_fx;                   // FP64 links in fixed point (dslash_fx64.cuh), or null
-    const void* N_fx;
-    int fx_exp[8];                      // their block exponents, [U, N][direction]
-    int fx_f1[4], fx_f0[4], fx_fe[4];   // temporal factors (ft1, bt1, ft3, bt3) in limbs, set by the launcher
     double r12_inv_scale;               // 1 / s for R12 fat links
     float lscale_u[9];                  // per-component scales of 16-bit fat links
     float lscale_n[9];                  // per-component scales of 16-bit Naik links
@@ -240,10 +235,16 @@ struct DslashArgs {
     int finish;
     double tol2;                        // FIN_RELIABLE: tol^2
     RedScratch red;
-    int run;                            // consecutive tiles a block takes (set by the launcher)
-    int red_defer;                      // 1: the blocks' sums are left to launch_red_finish (set by the launcher)
     double* red_out;                    // [vals] for FIN_STORE
     CgScalars* cg;                      // for FIN_CG_ALPHA / FIN_RELIABLE
+    int run;                            // consecutive tiles a block takes (set by the launcher)
+    int red_defer;                      // 1: the blocks' sums are left to launch_red_finish (set by the launcher)
+    int both;                           // 1: both parities in one launch (F64 fixed-point links, no reduction):
+                                        // in, out, x, y are parity-blocked full-lattice vectors
+    const void* U_fx;                   // FP64 links in fixed point (dslash_fx64.cuh), or null
+    const void* N_fx;
+    int fx_exp[8];                      // their block exponents, [U, N][direction]
+    int fx_f1[4], fx_f0[4], fx_fe[4];   // temporal factors (ft1, bt1, ft3, bt3) in limbs, set by the launcher
 };
 
 // Epilogue kinds (template parameter of the Dslash kernel)

@@ -1,10 +1,12 @@
-// Block partials plus a last-block finish, in a fixed order (deterministic).
+// Block partials and their sums, in a fixed order (deterministic).
 //
-// Every block writes one partial per reduced value to
-// partials[value * kMaxRedBlocks + blockIdx.x], fences, and bumps a counter;
-// the block that arrives last sums the partials of every value in a fixed
-// order (one warp per value, lane-strided, then a fixed shuffle tree), resets
-// the counter for the next launch and runs the finish logic.
+// Every block writes one partial per reduced value to partials[value * slots +
+// blockIdx.x]. In the vector kernels, and the Dslash of few blocks (slots =
+// kMaxRedBlocks), it then fences and bumps a counter; the block that arrives
+// last sums the partials of every value in a fixed order (one warp per value,
+// lane-strided, then a fixed shuffle tree), resets the counter for the next
+// launch and runs the finish logic. A Dslash of many blocks (slots =
+// kDeferSlots) leaves both to red_finish_kernel.
 #pragma once
 
 #include "hisq_internal.cuh"
@@ -67,7 +69,7 @@ __device__ __forceinline__ bool last_block_arrive(unsigned int* counter, unsigne
 
 // In the last block: out[v] = sum (or max, when is_max(v)) over slots of
 // partials[v][0 .. nslots). Must be called by all threads of the block.
-template <typename IsMax>
+template <int U = 1, typename IsMax>
 __device__ __forceinline__ void finish_values(const RedScratch& red, int nvals, int nslots,
                                               IsMax is_max, double* out_smem) {
     __threadfence();
@@ -78,15 +80,21 @@ __device__ __forceinline__ void finish_values(const RedScratch& red, int nvals, 
         const double* src = red.partials + (size_t)v * kMaxRedBlocks;
         const bool mx = is_max(v);
         double acc = 0.0;
-        // U loads in flight per lane: up to 4096 slots are summed while the
-        // rest of the GPU waits
-        constexpr int U = 8;
-        for (int i0 = lane; i0 < nslots; i0 += 32 * U) {
-            double t[U];
+        if (U > 1 && nslots > 64) {
+            // U loads in flight per lane: up to 4096 slots are summed while the
+            // rest of the GPU waits
+            for (int i0 = lane; i0 < nslots; i0 += 32 * U) {
+                double t[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) t[u] = i0 + 32 * u < nslots ? __ldcg(src + i0 + 32 * u) : 0.0;
+                for (int u = 0; u < U; ++u) t[u] = i0 + 32 * u < nslots ? __ldcg(src + i0 + 32 * u) : 0.0;
 #pragma unroll
-            for (int u = 0; u < U; ++u) acc = mx ? fmax(acc, t[u]) : acc + t[u];
+                for (int u = 0; u < U; ++u) acc = mx ? fmax(acc, t[u]) : acc + t[u];
+            }
+        } else {
+            for (int i = lane; i < nslots; i += 32) {
+                const double t = __ldcg(src + i);
+                acc = mx ? fmax(acc, t) : acc + t;
+            }
         }
         acc = mx ? warp_max(acc) : warp_sum(acc);
         if (lane == 0) out_smem[v] = acc;
