@@ -75,7 +75,7 @@ def test_operators(gpu_lib, n):
 # prec 0: FP64 inner iterations; 1 and 2: FP64 reliable updates; the solves' own tolerances
 @pytest.mark.parametrize("prec,n", [(0, 1), (0, 4), (1, 2), (1, 8), (2, 4)])
 def test_even_odd_solve(gpu_lib, prec, n):
-    L, m = (4, 6, 8, 10), 0.05
+    L, m = (4, 6, 4, 6), 0.1
     U, N = uneven_links(L, 55)
     b = gen.z2_source(L, n, seed=56)
     x, st = solve(gpu_lib, L, U, N, b, m, prec=prec, rn=18)
