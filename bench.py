@@ -187,8 +187,8 @@ class ClockSampler:
 # capture of that kernel (profiles/), keyed by (precision, lattice, n, rhs per
 # thread, min blocks, mapping flags). A mapping without a capture reports null.
 DSLASH_TRAFFIC = {
-    # profiles/dslash_bundle_f16_r18_r14_n8_48x48x48x12.md: 411.8 MB read + 54.6 MB written
-    ("f16", (48, 48, 48, 12), 8, 8, 4, 132): 466410496,
+    # profiles/dslash_bundle_f16_r18_r14_n8_48x48x48x12.md: 411.7 MB read + 54.4 MB written
+    ("f16", (48, 48, 48, 12), 8, 8, 4, 132): 466182656,
     # profiles/dslash_bundle_f32_r18_r14_n8_48x48x48x12.md: 824.4 MB read + 99.5 MB written
     ("f32", (48, 48, 48, 12), 8, 8, 3, 0): 923935488,
 }
